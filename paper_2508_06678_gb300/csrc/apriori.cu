@@ -31,33 +31,10 @@ using C2 = double2;
 struct Grid {
   Geom g{};
   FftPlan plan{};
-  int W = 2;
-  int col_threads = 128, row_threads = 256;
-  size_t col_smem = 0, row_smem = 0;
+  int W = 1;  // k_x columns per CTA of the column pass
+  size_t row_smem = 0;  // of the plainest launch shape: the grid is refused where that does not fit
   void* tw = nullptr;
 };
-
-FftPlan plan_of(int n) {
-  FftPlan p{};
-  p.n = n;
-  int m = n;
-  while (m % 8 == 0) { p.radix[p.npass++] = 8; m /= 8; }
-  if (m % 4 == 0) { p.radix[p.npass++] = 4; m /= 4; }
-  if (m % 2 == 0) { p.radix[p.npass++] = 2; m /= 2; }
-  while (m % 3 == 0) { p.radix[p.npass++] = 3; m /= 3; }
-  return p;
-}
-
-int threads_of(const FftPlan& p, int B, int floor_threads) {
-  int need = floor_threads;
-  for (int s = 0; s < p.npass; ++s) {
-    const int R = p.radix[s];
-    const int mi = R == 3 ? 2 : 8 / R;
-    const int t = ((p.n / R) * B + mi - 1) / mi;
-    if (t > need) need = t;
-  }
-  return (need + 31) / 32 * 32;
-}
 
 bool valid_n(int n) {
   if (n < 16 || n > 4096 || (n & 1)) return false;
@@ -76,13 +53,10 @@ void make_grid(Grid& G, int n, int K, double L, int nslot) {
   g.Ny = 2 * K + 1;
   g.SP = (g.Ny + 3) / 4 * 4;
   g.kscale = 2.0 * M_PI / L;
-  G.plan = plan_of(n);
-  G.W = 2;
-  G.col_threads = threads_of(G.plan, G.W, 128);
-  G.col_smem = (size_t)n * G.W * 16 + 2 * (size_t)G.W * g.Ny * 16;
+  G.plan = fft_plan(n, rt_elems(n, 8));
+  G.W = col_width(G.plan, 8);
   g.Kcp = (g.Kc + G.W - 1) / G.W * G.W;
   g.IP = g.Kcp;
-  G.row_threads = threads_of(G.plan, 1, 256);
   G.row_smem = (size_t)n * 16 + (size_t)(nslot > 2 ? nslot : 2) * n * 8;
 }
 
@@ -217,10 +191,10 @@ struct Ctx {
   cudaStream_t st = nullptr;
   cudaError_t err = cudaSuccess;
   void row(const Grid& G, RowDesc d) {
-    if (err == cudaSuccess) err = launch_row<double>(G.g, G.plan, d, G.tw, G.row_threads, G.row_smem, st);
+    if (err == cudaSuccess) err = launch_row<double>(G.g, G.plan, d, G.tw, st);
   }
   void col(const Grid& G, ColDesc d) {
-    if (err == cudaSuccess) err = launch_col<double>(G.g, G.plan, d, G.tw, G.W, G.col_threads, G.col_smem, st);
+    if (err == cudaSuccess) err = launch_col<double>(G.g, G.plan, d, G.tw, G.W, st);
   }
 };
 
@@ -229,6 +203,7 @@ ColDesc col_desc(double U, const qg_closure* cl, int test_m2max) {
   d.U = U;
   d.test_ratio = cl->test_ratio;
   d.test_m2max = test_m2max;
+  d.test_kmax = 1 << 30;  // the scratch arrays hold other fields before: every column is written
   const int p = (cl->kind == QG_SMAG || cl->kind == QG_DSMAG) ? 2 : 3;
   d.closure_pow = p;
   d.rpow = std::pow(cl->test_ratio, p);
@@ -276,7 +251,7 @@ extern "C" int qg_sgs_apriori(const double* omega_fr, int32_t n_fr, int32_t n_le
   int dev = 0, optin = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (F.col_smem > (size_t)optin - 1024 || F.row_smem > (size_t)optin - 1024 || Cg.row_smem > (size_t)optin - 1024) {
+  if (2 * (size_t)n_fr * 16 + 4 * (size_t)F.g.Ny * 16 > (size_t)optin - 1024 || F.row_smem > (size_t)optin - 1024 || Cg.row_smem > (size_t)optin - 1024) {
     qg::set_last_error("qg_sgs_apriori: grid too large for the kernels' shared memory");
     return QG_ERR_UNSUPPORTED;
   }
@@ -288,15 +263,18 @@ extern "C" int qg_sgs_apriori(const double* omega_fr, int32_t n_fr, int32_t n_le
   auto phys = [&](int n) { return pool.get((size_t)n * n * 8); };
   // twiddles per grid size
   for (Grid* G : {&F, &Cg, &Cf}) {
-    std::vector<double> tw(2 * (size_t)G->g.n);
-    for (int j = 0; j < G->g.n; ++j) {
+    std::vector<double> tw(2 * (size_t)G->plan.table);
+    for (int e = 0; e < G->plan.table; ++e) {
       double c, s;
-      cos_sin_frac(j, G->g.n, &c, &s);
-      tw[2 * j] = c;
-      tw[2 * j + 1] = -s;
+      cos_sin_frac(fft_table_exponent(G->plan, e), G->g.n, &c, &s);
+      tw[2 * e] = c;
+      tw[2 * e + 1] = -s;
     }
+    // twiddles, then the wavenumbers 2 pi m / L
+    for (int m = 0; m <= G->g.n / 2; ++m) tw.push_back(G->g.kscale * m);
     G->tw = pool.get(tw.size() * 8);
     if (G->tw) cudaMemcpy(G->tw, tw.data(), tw.size() * 8, cudaMemcpyHostToDevice);
+    G->g.kt = static_cast<const double*>(G->tw) + 2 * (size_t)G->plan.table;
   }
   const size_t nf2 = (size_t)n_fr * n_fr, nc2 = (size_t)n_les * n_les;
   void* Pw = phys(n_fr);
@@ -498,17 +476,15 @@ extern "C" int qg_sgs_apriori(const double* omega_fr, int32_t n_fr, int32_t n_le
     int nd = 0;
     const int b4[4] = {D_U, D_V, D_WX, D_WY};
     for (int i = 0; i < 4; ++i) c.der[nd++] = b4[i];
-    if (smag) { c.der[nd++] = D_PXY; c.der[nd++] = D_PD; }
-    if (dyn) {
-      for (int i = 0; i < 4; ++i) c.der[nd++] = b4[i] | D_TEST;
-      if (smag) { c.der[nd++] = D_PXY | D_TEST; c.der[nd++] = D_PD | D_TEST; }
-    }
+    if (smag) c.der[2] = D_W;
+    if (dyn)
+      for (int i = 0; i < 4; ++i) c.der[nd++] = c.der[i] | D_TEST;
     c.nder = nd;
     for (int i = 0; i < nd; ++i) c.dout[i] = Mc[i];
     cx.col(Cg, c);
     RowDesc r{};
     r.prog = kind == QG_SMAG ? RP_SMAG : kind == QG_LEITH ? RP_LEITH : kind == QG_DSMAG ? RP_DSMAG : RP_DLEITH;
-    r.nin = nd;
+    r.nin = smag ? (dyn ? 12 : 6) : nd;
     r.nout = dyn ? 6 : 3;
     r.dx_mask = dyn ? 0x12u : 0x2u;
     for (int i = 0; i < nd; ++i) r.in[i] = Mc[i];
@@ -606,22 +582,25 @@ extern "C" int qg_grid_filter(const double* omega_fr, int32_t nsnap, int32_t n_f
   int dev = 0, optin = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (F.col_smem > (size_t)optin - 1024 || F.row_smem > (size_t)optin - 1024) {
+  if (2 * (size_t)n_fr * 16 + 4 * (size_t)F.g.Ny * 16 > (size_t)optin - 1024 || F.row_smem > (size_t)optin - 1024) {
     qg::set_last_error("qg_grid_filter: grid too large for the kernels' shared memory");
     return QG_ERR_UNSUPPORTED;
   }
   Pool pool;
   Ctx cx;
   for (Grid* G : {&F, &Cg}) {
-    std::vector<double> tw(2 * (size_t)G->g.n);
-    for (int j = 0; j < G->g.n; ++j) {
+    std::vector<double> tw(2 * (size_t)G->plan.table);
+    for (int e = 0; e < G->plan.table; ++e) {
       double c, s;
-      cos_sin_frac(j, G->g.n, &c, &s);
-      tw[2 * j] = c;
-      tw[2 * j + 1] = -s;
+      cos_sin_frac(fft_table_exponent(G->plan, e), G->g.n, &c, &s);
+      tw[2 * e] = c;
+      tw[2 * e + 1] = -s;
     }
+    // twiddles, then the wavenumbers 2 pi m / L
+    for (int m = 0; m <= G->g.n / 2; ++m) tw.push_back(G->g.kscale * m);
     G->tw = pool.get(tw.size() * 8);
     if (G->tw) cudaMemcpy(G->tw, tw.data(), tw.size() * 8, cudaMemcpyHostToDevice);
+    G->g.kt = static_cast<const double*>(G->tw) + 2 * (size_t)G->plan.table;
   }
   const size_t nf2 = (size_t)n_fr * n_fr, nc2 = (size_t)n_les * n_les;
   void* Pw = pool.get(nf2 * 8);

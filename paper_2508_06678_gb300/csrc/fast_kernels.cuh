@@ -1,7 +1,7 @@
-// Specialised row / column passes on the register-resident engines (E16 for N = 2^p, E12 for N = 3 * 2^p).
-// Same arithmetic and data layouts as row.cu / column.cu (see there for the
-// equations); only the FFT organisation differs.  Included by fast_<N>.cu,
-// one translation unit per grid size.
+// Row / column passes of the large FP32 grids, specialised for one N at compile time.  Same arithmetic and data
+// layouts as row_kernel.cuh / column_kernel.cuh (see there for the equations); a row's or a column's transforms run
+// one after another and keep everything between them in registers.  Included by grid_<N>.cu, one translation unit
+// per grid size.
 #pragma once
 
 #include <atomic>
@@ -10,9 +10,6 @@
 #include "qg_kernels.h"
 #include "tma.cuh"
 
-#ifndef QG_ROW_MINB
-#define QG_ROW_MINB 4
-#endif
 #ifndef QG_COL_MINB
 #define QG_COL_MINB 2
 #endif
@@ -33,36 +30,44 @@ namespace qg {
 namespace fast {
 
 template <int N> struct RowCfg {
-  static constexpr int TT = N / elems_per_thread(N);
-  static constexpr int ROWS = TT >= QG_ROW_CTA_THREADS ? 1 : QG_ROW_CTA_THREADS / TT;
+  static constexpr int TT = Eng<float, N>::TT;
+  // whole rows, a divisor of N, filling at most QG_ROW_CTA_THREADS threads
+  static constexpr int rows(int r) { return r <= 1 ? 1 : N % r == 0 ? r : rows(r - 1); }
+  static constexpr int ROWS = rows(QG_ROW_CTA_THREADS / TT);
   static constexpr int THREADS = TT * ROWS;
 };
-// resident CTAs per SM requested from the register allocator (FP32; FP64 takes 1)
-template <typename T, int OP = -1> struct Occ {
-  static constexpr int row = QG_ROW_MINB * 128 / QG_ROW_CTA_THREADS > 0 ? QG_ROW_MINB * 128 / QG_ROW_CTA_THREADS : 1;
-  static constexpr int col = OP == CO_DYN_REDUCE ? QG_COL_MINB_REDUCE
-                             : (OP == CO_FORWARD || OP == CO_FORWARD2 || OP == CO_FORWARD_N ||
-                                OP == CO_AB2CN_FINAL) ? QG_COL_MINB_FWD
-                             : OP == CO_CURL    ? QG_COL_MINB_CURL
-                                                : QG_COL_MINB;
+// Resident CTAs per SM requested from the register allocator: 512 threads an SM leave each thread 128 registers, which
+// the row programs and the column ops need (384 with eighteen elements per thread).  Asking for four row CTAs and two
+// column CTAs whatever their size left 64 registers at 4096^2, and a Leith step there took 2.06 ms instead of 1.39.
+template <int N> constexpr int row_occ() {
+  const int target = Eng<float, N>::EL == 18 ? 384 : 512;
+  return target / RowCfg<N>::THREADS > 0 ? target / RowCfg<N>::THREADS : 1;
+}
+template <int N> constexpr int col_threads();
+template <int OP, int N> struct Occ {
+  static constexpr int want = OP == CO_DYN_REDUCE ? QG_COL_MINB_REDUCE
+                              : (OP == CO_FORWARD || OP == CO_FORWARD2 || OP == CO_FORWARD_N ||
+                                 OP == CO_AB2CN_FINAL) ? QG_COL_MINB_FWD
+                              : OP == CO_CURL    ? QG_COL_MINB_CURL
+                                                 : QG_COL_MINB;
+  static constexpr int most = 512 / col_threads<N>() > 0 ? 512 / col_threads<N>() : 1;
+  static constexpr int col = want < most ? want : most;
 };
-template <int OP> struct Occ<double, OP> { static constexpr int row = 1, col = 1; };
 
-#ifndef QG_COL_W
-#define QG_COL_W 2
-#endif
 template <int N> struct ColCfg {
-  static constexpr int W = QG_COL_W;  // k_x columns per CTA
-  static constexpr int TT = N / elems_per_thread(N);
-  static constexpr int THREADS = W * TT;
+  static constexpr int W = kFastWidth;  // k_x columns per CTA
+  static constexpr int TT = Eng<float, N>::TT;
+  static constexpr bool ALL = W * TT % 32 == 0;          // no idle threads fill up the last warp
+  static constexpr int THREADS = (W * TT + 31) / 32 * 32;
   // column stride in shared memory (complex elements): 16 / W mod 16 keeps the exchanges conflict-free
-  static constexpr int CP = N + N / 16 + 16 / W;
+  static constexpr int CP = (N + N / 16 + 15) / 16 * 16 + 16 / W;
   static constexpr int BR = fast_box_rows(N);  // rows per TMA box
-  static constexpr int NBOX = N / BR;
+  static constexpr int NBOX = (N + BR - 1) / BR;
 };
+template <int N> constexpr int col_threads() { return ColCfg<N>::THREADS; }
 // bytes of one shared-memory stage: a dense W x N tile for TMA, or W padded exchange columns
 template <typename T, int N> __host__ __device__ constexpr int col_stage_bytes() {
-  constexpr int dense = N * ColCfg<N>::W * 2 * (int)sizeof(T);
+  constexpr int dense = ColCfg<N>::NBOX * ColCfg<N>::BR * ColCfg<N>::W * 2 * (int)sizeof(T);
   constexpr int padded = ColCfg<N>::W * ColCfg<N>::CP * 2 * (int)sizeof(T);
   return ((dense > padded ? dense : padded) + 1023) / 1024 * 1024;
 }
@@ -77,8 +82,7 @@ template <typename T, int N> constexpr bool lean_fits() {
 #define QG_PACKED_COL_MASK 0xFED7
 #endif
 template <int OP> constexpr bool col_packed() { return (QG_PACKED_COL_MASK >> OP) & 1; }
-// bounded device waits: about one second of SM clocks
-constexpr long long kWaitCycles = 2000000000LL;
+using tma::kWaitCycles;
 
 template <typename T>
 __device__ __forceinline__ void leith_p(T u, T v, T wx, T wy, T& J, T& P, T& Q) {
@@ -112,30 +116,40 @@ struct RowCtx {
   const Geom* g;
   int bad;
 
-  // inverse x-transform of the pair (A + i B) of half-spectrum rows; B may be null
-  __device__ __forceinline__ void inv_pair(C* x, const void* Av, const void* Bv) {
-    const C* A = reinterpret_cast<const C*>(Av) + (size_t)y * g->IP;
-    const C* B = Bv ? reinterpret_cast<const C*>(Bv) + (size_t)y * g->IP : nullptr;
+  // inverse x-transform of the pair a + i b of half-spectrum rows given by f(k, a, b), k <= K
+  template <typename F> __device__ __forceinline__ void inv_pair_of(C* x, F f) {
 #pragma unroll
     for (int m = 0; m < E::EL; ++m) {
       const int k = t + TT * m;
-      C z = mk<C>(T(0), T(0));
+      C z = mk<C>(T(0), T(0)), a, b;
       if (k <= E::K) {
-        C a = A[k];
-        C b = B ? B[k] : mk<C>(T(0), T(0));
+        f(k, a, b);
         if (k == 0) {
           a.y = T(0);
           b.y = T(0);
         }
         z = mk<C>(a.x - b.y, a.y + b.x);
       } else if (k >= N - E::K) {
-        const C a = A[N - k];
-        const C b = B ? B[N - k] : mk<C>(T(0), T(0));
+        f(N - k, a, b);
         z = mk<C>(a.x + b.y, b.x - a.y);
       }
       x[m] = z;
     }
     E::run(x, t, b0, b1, ph, tw, +1);
+  }
+
+  __device__ __forceinline__ const C* mixed_row(const void* A) const {
+    return reinterpret_cast<const C*>(A) + (size_t)y * g->IP;
+  }
+
+  // inverse x-transform of the pair (A + i B) of half-spectrum rows; B may be null
+  __device__ __forceinline__ void inv_pair(C* x, const void* Av, const void* Bv) {
+    const C* A = mixed_row(Av);
+    const C* B = Bv ? mixed_row(Bv) : nullptr;
+    inv_pair_of(x, [&](int k, C& a, C& b) {
+      a = A[k];
+      b = B ? B[k] : mk<C>(T(0), T(0));
+    });
   }
 
   // forward x-transform of (re, im) = two real rows, split, optional i k_x, store kept columns
@@ -184,6 +198,12 @@ struct RowCtx {
 // One level of the stage products: inverse-transform (u, v), (w_x, w_y)
 // [and (psi_xy, psi_xx - psi_yy)] and form J = u w_x + v w_y, P = g w_x,
 // Q = g w_y with g = |grad w| (Leith) or |S| (Smagorinsky); NONE forms J only.
+// The Smagorinsky programs read the four mixed fields u, v, w, w_y of a level:
+// in mixed space (k_x, y) the derivatives in x are factors, so w_x = i k_x w and,
+// with u = -psi_y + U, v = psi_x and psi_yy = w - psi_xx, the strain pair is
+// psi_xy = -i k_x u (the mean U sits at k_x = 0) and psi_xx - psi_yy = 2 i k_x v - w.
+// Two fields fewer per level leave the column pass (a third of its inverse
+// transforms and stores) than with the strain pair stored.
 template <typename T, int N, bool SMAG, bool NONE>
 __device__ __forceinline__ void level_products(RowCtx<T, N>& cx, cplx_t<T>* x, const void* const* in, T* J, T* P,
                                                T* Q) {
@@ -195,10 +215,19 @@ __device__ __forceinline__ void level_products(RowCtx<T, N>& cx, cplx_t<T>* x, c
     J[m] = x[m].x;  // u_total
     P[m] = x[m].y;  // v
   }
-  cx.inv_pair(x, in[2], in[3]);  // (w_x, w_y)
   if constexpr (SMAG) {
+    const T ks = T(cx.g->kscale);
+    const C *u = cx.mixed_row(in[0]), *v = cx.mixed_row(in[1]), *w = cx.mixed_row(in[2]), *wy = cx.mixed_row(in[3]);
+    cx.inv_pair_of(x, [&](int k, C& a, C& b) {  // (w_x, w_y)
+      a = cmul_ik(w[k], ks * T(k));
+      b = wy[k];
+    });
     C s[E::EL];
-    cx.inv_pair(s, in[4], in[5]);
+    cx.inv_pair_of(s, [&](int k, C& a, C& b) {  // (psi_xy, psi_xx - psi_yy)
+      const T kx = ks * T(k);
+      a = cmul_ik(u[k], -kx);
+      b = csub(cmul_ik(v[k], T(2) * kx), w[k]);
+    });
 #pragma unroll
     for (int m = 0; m < E::EL; ++m) {
       T j, p, q;
@@ -208,9 +237,11 @@ __device__ __forceinline__ void level_products(RowCtx<T, N>& cx, cplx_t<T>* x, c
       Q[m] = q;
     }
   } else if constexpr (NONE) {
+    cx.inv_pair(x, in[2], in[3]);  // (w_x, w_y)
 #pragma unroll
     for (int m = 0; m < E::EL; ++m) J[m] = J[m] * x[m].x + P[m] * x[m].y;
   } else {
+    cx.inv_pair(x, in[2], in[3]);  // (w_x, w_y)
 #pragma unroll
     for (int m = 0; m < E::EL; ++m) {
       T j, p, q;
@@ -228,7 +259,7 @@ __device__ __forceinline__ void level_products(RowCtx<T, N>& cx, cplx_t<T>* x, c
 }
 
 template <typename T, int N, int PROG>
-__global__ void __launch_bounds__(RowCfg<N>::THREADS, Occ<T>::row) row_fast_kernel(Geom g, RowDesc d,
+__global__ void __launch_bounds__(RowCfg<N>::THREADS, row_occ<N>()) row_fast_kernel(Geom g, RowDesc d,
                                                                        const cplx_t<T>* __restrict__ tw) {
   pdl_enter();
   using E = Eng<T, N>;
@@ -257,7 +288,7 @@ __global__ void __launch_bounds__(RowCfg<N>::THREADS, Occ<T>::row) row_fast_kern
     constexpr bool smag = PROG == RP_SMAG || PROG == RP_DSMAG;
     constexpr bool dyn = PROG == RP_DLEITH || PROG == RP_DSMAG;
     constexpr bool none = PROG == RP_NONE;
-    constexpr int per = smag ? 6 : 4;  // inputs per level
+    constexpr int per = 4;  // inputs per level
     T J[E::EL], P[E::EL], Q[E::EL];
     level_products<T, N, smag, none>(cx, x, d.in + 0, J, P, Q);
     if constexpr (none) {
@@ -476,7 +507,7 @@ constexpr int kStateBatch = QG_STATE_BATCH;
 // and the tiles come through one TMA stage, so three CTAs fit on an SM.  The launcher picks it when that turns
 // a partial second wave of column CTAs into one wave.
 template <typename T, int N, int OP, bool LEAN = false>
-__global__ void __launch_bounds__(ColCfg<N>::THREADS, LEAN ? 3 : Occ<T, OP>::col) col_fast_kernel(
+__global__ void __launch_bounds__(ColCfg<N>::THREADS, LEAN ? 3 : Occ<OP, N>::col) col_fast_kernel(
     Geom g, ColDesc d, const cplx_t<T>* __restrict__ tw, const __grid_constant__ TmaSet tm) {
   pdl_enter();
   using E = Eng<T, N>;
@@ -489,7 +520,7 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, LEAN ? 3 : Occ<T, OP>::col
   constexpr int BR = ColCfg<N>::BR;
   constexpr int NBOX = ColCfg<N>::NBOX;
   constexpr int SB = col_stage_bytes<T, N>();
-  constexpr uint32_t FIELD_BYTES = (uint32_t)N * W * 2 * sizeof(T);
+  constexpr uint32_t FIELD_BYTES = (uint32_t)NBOX * BR * W * 2 * sizeof(T);
   // shared memory: exchange buffer | stage 0 | stage 1.  A stage receives a
   // field's dense W x N tile by TMA, then serves as the FFT's second exchange
   // buffer, and in the inverse phase holds the dense output tile for the TMA store.
@@ -502,10 +533,12 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, LEAN ? 3 : Occ<T, OP>::col
   C* xbuf = reinterpret_cast<C*>(sbase);
   C* stage[2] = {reinterpret_cast<C*>(sbase + SB), reinterpret_cast<C*>(sbase + (NSTG == 2 ? 2 : 1) * SB)};
   const int c = threadIdx.x % W;
-  const int t = threadIdx.x / W;
+  // the idle threads that fill up the last warp keep the barriers; they neither store nor add to a sum
+  const bool act = ColCfg<N>::ALL || (int)threadIdx.x / W < TT;
+  const int t = act ? threadIdx.x / W : 0;
   const int mx = blockIdx.x * W + c;
   const int c0 = blockIdx.x * W;
-  const bool col_ok = mx < E::Kc;
+  const bool col_ok = mx < E::Kc && act;
   const bool lead = threadIdx.x == 0;
   int ph = 0;
   const C* twb = tw;
@@ -564,7 +597,7 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, LEAN ? 3 : Occ<T, OP>::col
 #pragma unroll
       for (int m = 0; m < E::EL; ++m) x[m] = st[(t + TT * m) * W + c];
       ph = 0;
-      E::template run<col_packed<OP>()>(x, t, xbuf + c * CP, st + c * CP, ph, twb, -1);
+      E::template run<col_packed<OP>()>(x, t, xbuf + c * CP, st + c * CP, ph, twb, -1, act);
       // every thread is done with this stage: hand it to the TMA for field f + NSTG
       tma::fence_proxy_async();
       __syncthreads();
@@ -582,7 +615,7 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, LEAN ? 3 : Occ<T, OP>::col
         C* s0 = reinterpret_cast<C*>(d.scr[0]);
         C* s1 = reinterpret_cast<C*>(d.scr[1]);
         C* s2 = reinterpret_cast<C*>(d.scr[2]);
-        constexpr int LB = QG_LEAN_BATCH;
+        constexpr int LB = E::EL % QG_LEAN_BATCH == 0 ? QG_LEAN_BATCH : 6;
         static_assert(E::EL % LB == 0, "the load batch must divide the thread's elements");
 #pragma unroll
         for (int m0 = 0; m0 < E::EL; m0 += LB) {
@@ -604,7 +637,7 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, LEAN ? 3 : Occ<T, OP>::col
           for (int q = 0; q < LB; ++q) {
             const int m = m0 + q;
             const int k = t + TT * m;
-            if (!(k <= K || k >= N - K)) continue;
+            if (!(k <= K || k >= N - K) || !act) continue;
             const int my = k <= K ? k : k - N;
             const T ky = T(g.kscale) * T(my);
             const size_t gi = colbase + (k <= K ? k : k - N + Ny);
@@ -649,7 +682,7 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, LEAN ? 3 : Occ<T, OP>::col
           else if (f == 1) B[m] = X;
           else B[m] = cadd(B[m], cmul_ik(X, ky));
         } else if constexpr (OP == CO_DYN_REDUCE) {
-          const bool kept = k <= K || k >= N - K;
+          const bool kept = (k <= K || k >= N - K) && act;
           const int r = k <= K ? k : k - N + Ny;
           const bool in_test = mx * mx + my * my <= d.test_m2max;
           if (f == 0) {
@@ -769,7 +802,7 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, LEAN ? 3 : Occ<T, OP>::col
     const C* bhp = reinterpret_cast<const C*>(d.bh);
     C* ep = reinterpret_cast<C*>(d.eprev);
     C* wsp = reinterpret_cast<C*>(d.wss);
-    constexpr int GB = E::EL % kStateBatch == 0 ? kStateBatch : 4;  // a divisor of the thread's elements
+    constexpr int GB = E::EL % kStateBatch == 0 ? kStateBatch : E::EL % 4 == 0 ? 4 : 6;  // a divisor of the thread's elements
     static_assert(E::EL % GB == 0, "state batch must divide the elements per thread");
 #pragma unroll
     for (int m0 = 0; m0 < E::EL; m0 += GB) {
@@ -973,10 +1006,12 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, LEAN ? 3 : Occ<T, OP>::col
       // at most the previous field's store is still reading (its tile is in neither exchange buffer)
       if (lead) tma::wait_group_read<1>();
       ph = 0;
-      E::template run<col_packed<OP>()>(x, t, b0 + c * CP, b1 + c * CP, ph, twb, +1);
+      E::template run<col_packed<OP>()>(x, t, b0 + c * CP, b1 + c * CP, ph, twb, +1, act);
       // the tile buffer's last reads in this transform came before its last exchange's barrier
+      if (act) {
 #pragma unroll
-      for (int m = 0; m < E::EL; ++m) st[(t + TT * m) * W + c] = x[m];
+        for (int m = 0; m < E::EL; ++m) st[(t + TT * m) * W + c] = x[m];
+      }
       tma::fence_proxy_async();
       __syncthreads();
       t2 = t1;
@@ -1087,13 +1122,9 @@ cudaError_t launch_col_fast(const Geom& g, const ColDesc& d, const void* tw, con
 #undef QG_COL_CASE
 }
 
-#define QG_INSTANTIATE_FAST(N)                                                                          \
-  template <> int fast_col_width<N>() { return fast::ColCfg<N>::W; }                                    \
+#define QG_INSTANTIATE_FAST(N)                                                                            \
   template cudaError_t launch_row_fast<float, N>(const Geom&, const RowDesc&, const void*, cudaStream_t);  \
-  template cudaError_t launch_row_fast<double, N>(const Geom&, const RowDesc&, const void*, cudaStream_t); \
-  template cudaError_t launch_col_fast<float, N>(const Geom&, const ColDesc&, const void*, const TmaSet&,       \
-                                                 cudaStream_t);                                             \
-  template cudaError_t launch_col_fast<double, N>(const Geom&, const ColDesc&, const void*, const TmaSet&,      \
-                                                  cudaStream_t);
+  template cudaError_t launch_col_fast<float, N>(const Geom&, const ColDesc&, const void*, const TmaSet&,  \
+                                                 cudaStream_t);
 
 }  // namespace qg

@@ -1,4 +1,4 @@
-// Specialised passes for N = 1024 (power of two); see fast_kernels.cuh.
+// FP32 passes of the 1024 x 1024 grid; see fast_kernels.cuh.
 #include "fast_kernels.cuh"
 
 namespace qg {

@@ -1,4 +1,4 @@
-// Specialised passes for N = 2048 (power of two); see fast_kernels.cuh.
+// FP32 passes of the 2048 x 2048 grid; see fast_kernels.cuh.
 #include "fast_kernels.cuh"
 
 namespace qg {

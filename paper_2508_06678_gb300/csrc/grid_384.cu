@@ -1,4 +1,4 @@
-// Specialised passes for N = 384 (3 * 2^p, engine E12); see fast_kernels.cuh.
+// FP32 passes of the 384 x 384 grid; see fast_kernels.cuh.
 #include "fast_kernels.cuh"
 
 namespace qg {

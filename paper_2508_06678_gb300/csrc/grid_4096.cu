@@ -1,4 +1,4 @@
-// Specialised passes for N = 4096 (power of two); see fast_kernels.cuh.
+// FP32 passes of the 4096 x 4096 grid; see fast_kernels.cuh.
 #include "fast_kernels.cuh"
 
 namespace qg {

@@ -1,4 +1,4 @@
-// Specialised passes for N = 512 (power of two); see fast_kernels.cuh.
+// FP32 passes of the 512 x 512 grid; see fast_kernels.cuh.
 #include "fast_kernels.cuh"
 
 namespace qg {

@@ -54,35 +54,15 @@ bool valid_n(int n) {
   return m == 1;
 }
 
-FftPlan plan_for(int n) {
-  FftPlan p{};
-  p.n = n;
-  int m = n;
-  while (m % 8 == 0) { p.radix[p.npass++] = 8; m /= 8; }
-  if (m % 4 == 0) { p.radix[p.npass++] = 4; m /= 4; }
-  if (m % 2 == 0) { p.radix[p.npass++] = 2; m /= 2; }
-  while (m % 3 == 0) { p.radix[p.npass++] = 3; m /= 3; }
-  return p;
-}
-
-int threads_for(const FftPlan& p, int B, int floor_threads) {
-  int need = floor_threads;
-  for (int s = 0; s < p.npass; ++s) {
-    const int R = p.radix[s];
-    const int mi = R == 3 ? 2 : 8 / R;
-    const int t = ((p.n / R) * B + mi - 1) / mi;
-    if (t > need) need = t;
-  }
-  return (need + 31) / 32 * 32;
-}
-
-// twiddle table exp(-2 pi i j / n) written on the device (CUDA's sincospi)
+// the plan's twiddle table exp(-2 pi i j / n) written on the device (CUDA's sincospi)
+// (and the wavenumbers 2 pi m / L, FP64)
 template <typename T>
-__global__ void twiddle_kernel(cplx_t<T>* tw, int n) {
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
+__global__ void twiddle_kernel(cplx_t<T>* tw, FftPlan plan, double* kt, double kscale) {
+  for (int m = blockIdx.x * blockDim.x + threadIdx.x; m <= plan.n / 2; m += gridDim.x * blockDim.x) kt[m] = kscale * m;
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < plan.table; e += gridDim.x * blockDim.x) {
     double s, c;
-    sincospi(2.0 * double(j) / double(n), &s, &c);
-    tw[j] = mk<cplx_t<T>>(T(c), T(-s));
+    sincospi(2.0 * double(fft_table_exponent(plan, e)) / double(plan.n), &s, &c);
+    tw[e] = mk<cplx_t<T>>(T(c), T(-s));
   }
 }
 
@@ -117,14 +97,10 @@ int run_stats(const void* omega, int n, double L, cudaStream_t st, double* stats
   g.Ny = 2 * g.K + 1;
   g.SP = (g.Ny + 3) / 4 * 4;
   g.kscale = 2.0 * M_PI / L;
-  const FftPlan plan = plan_for(n);
-  const int W = sizeof(T) == 4 ? 4 : 2;
+  const FftPlan plan = fft_plan(n, rt_elems(n, sizeof(T)));
+  const int W = col_width(plan, sizeof(T));
   g.Kcp = (g.Kc + W - 1) / W * W;
   g.IP = g.Kcp;
-  const int col_threads = threads_for(plan, W, 128);
-  const size_t col_smem = (size_t)n * W * csz + 2 * (size_t)W * g.Ny * csz;
-  const int row_threads = threads_for(plan, 1, 256);
-  const size_t row_smem = (size_t)n * csz + 2 * (size_t)n * esz;
 
   // scratch layout
   const size_t b_mixed = align256((size_t)n * g.IP * csz);
@@ -133,7 +109,8 @@ int run_stats(const void* omega, int n, double L, cudaStream_t st, double* stats
   const size_t b_tw = align256((size_t)n * csz);
   const int nred = 512;
   const size_t b_red = align256((size_t)2 * nred * sizeof(double));
-  const size_t need = b_mixed + b_spec + b_phys + b_tw + b_red;
+  const size_t b_kt = align256((size_t)(n / 2 + 1) * sizeof(double));
+  const size_t need = b_mixed + b_spec + b_phys + b_tw + b_red + b_kt;
   if (need > kScratchBytes)
     return na_fail(QG_ERR_ARG, "qg_field_stats_static: n=%d needs %zu scratch bytes, the array holds %zu", n, need,
                    kScratchBytes);
@@ -142,9 +119,11 @@ int run_stats(const void* omega, int n, double L, cudaStream_t st, double* stats
   unsigned char* phys = spec + b_spec;
   unsigned char* tw = phys + b_phys;
   double* red = reinterpret_cast<double*>(tw + b_tw);
+  double* kt = reinterpret_cast<double*>(tw + b_tw + b_red);
+  g.kt = kt;
 
   // the spectral scratch starts at zero (its padding columns are never written)
-  twiddle_kernel<T><<<(n + 255) / 256, 256, 0, st>>>(reinterpret_cast<cplx_t<T>*>(tw), n);
+  twiddle_kernel<T><<<(n + 255) / 256, 256, 0, st>>>(reinterpret_cast<cplx_t<T>*>(tw), plan, kt, g.kscale);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaMemsetAsync(spec, 0, b_spec, st);
   if (e != cudaSuccess) return na_fail(QG_ERR_CUDA, "qg_field_stats_static: setup: %s", cudaGetErrorString(e));
@@ -157,7 +136,7 @@ int run_stats(const void* omega, int n, double L, cudaStream_t st, double* stats
   r.in_phys = 1;
   r.phys_in = omega;
   r.out[0] = mixed;
-  e = launch_row<T>(g, plan, r, tw, row_threads, row_smem, st);
+  e = launch_row<T>(g, plan, r, tw, st);
   if (e != cudaSuccess) return na_fail(QG_ERR_CUDA, "qg_field_stats_static: row pass: %s", cudaGetErrorString(e));
   ColDesc c{};
   c.op = CO_FORWARD;
@@ -171,7 +150,7 @@ int run_stats(const void* omega, int n, double L, cudaStream_t st, double* stats
   c.der[0] = D_W;
   c.dout[0] = mixed;  // each CTA reads its own columns before writing them
   c.test_ratio = 2.0;
-  e = launch_col<T>(g, plan, c, tw, W, col_threads, col_smem, st);
+  e = launch_col<T>(g, plan, c, tw, W, st);
   if (e != cudaSuccess) return na_fail(QG_ERR_CUDA, "qg_field_stats_static: column pass: %s", cudaGetErrorString(e));
   // physical field of the projected state
   RowDesc r2{};
@@ -181,7 +160,7 @@ int run_stats(const void* omega, int n, double L, cudaStream_t st, double* stats
   r2.in[0] = mixed;
   r2.out_phys = 1;
   r2.phys_out = phys;
-  e = launch_row<T>(g, plan, r2, tw, row_threads, row_smem, st);
+  e = launch_row<T>(g, plan, r2, tw, st);
   if (e != cudaSuccess) return na_fail(QG_ERR_CUDA, "qg_field_stats_static: row pass: %s", cudaGetErrorString(e));
   // energy, enstrophy (FP64 Parseval sums) and max |w|, finiteness
   e = launch_spectral_sums<T>(g, spec, red, nred, stats, st);

@@ -1,0 +1,81 @@
+// Host side of the run-time FFT engine (fft.cuh): plans, and the launch shapes of the passes that use it.
+#include "qg_kernels.h"
+
+namespace qg {
+
+FftPlan fft_plan(int n, int el) {
+  FftPlan p;
+  p.n = n;
+  p.el = el;
+  const Radices r = fft_radices(n, p.el);
+  p.tt = n / p.el;
+  p.npass = r.np;
+  for (int i = 0; i < p.npass; ++i)
+    p.pass[i] = {r.radix[i], r.ns[i], r.ns[i] > 1 ? (unsigned)((1ull << 32) / (unsigned)r.ns[i] + 1) : 0u, r.off[i]};
+  p.table = r.table;
+  p.buf = n + n / 16 + 1;
+  return p;
+}
+
+// dynamic shared memory a CTA can have: 227 KB less the passes' static part (under 768 bytes)
+constexpr size_t kSmemCap = 227 * 1024 - 768;
+
+RowConfig row_config(const FftPlan& p, const RowDesc& d, int esz) {
+  RowConfig c{};
+  const bool direct = d.prog == RP_SCALE || d.prog == RP_COPY;
+  int nin = d.nin, nout = d.nout;
+  if (direct) nin = nout = d.npair > 0 ? 2 * d.npair : d.in_phys ? d.nout : d.nin;
+  c.nslot = direct ? 0 : (nin > nout ? nin : nout);
+  auto tasks = [](int rows, int nf) { return rows * (nf / 2) + (nf & 1 ? (rows + 1) / 2 : 0); };
+  auto bytes = [&](int rows, int groups, int nbuf) {
+    return (size_t)groups * nbuf * p.buf * 2 * esz + (size_t)rows * c.nslot * p.n * esz;
+  };
+  const bool odd = (nin & 1) || (nout & 1);
+  c.rows = odd && (direct || (p.n >= 256 && bytes(2, 1, 2) <= kSmemCap / 2)) ? 2 : 1;
+  const int most = tasks(c.rows, nin) > tasks(c.rows, nout) ? tasks(c.rows, nin) : tasks(c.rows, nout);
+  const int target = esz == 4 ? 256 : 192;
+  int groups = target / p.tt;
+  if (groups < 1) groups = 1;
+  if (groups > most) groups = most;
+  // even rounds
+  const int rounds = (most + groups - 1) / groups;
+  groups = (most + rounds - 1) / rounds;
+  while (groups > 1 && bytes(c.rows, groups, 2) > kSmemCap / 2) --groups;
+  c.groups = groups;
+  c.one_buf = bytes(c.rows, groups, 2) > kSmemCap;
+  if (c.rows == 2 && bytes(2, groups, 1) > kSmemCap) c.rows = 1;
+  c.smem = bytes(c.rows, groups, c.one_buf ? 1 : 2);
+  c.threads = (groups * p.tt + 31) / 32 * 32;
+  c.warp = p.tt <= 32 && 32 % p.tt == 0;
+  return c;
+}
+
+int col_width(const FftPlan& p, int esz) {
+  if (p.n <= 512) return 1;
+  return esz == 4 && 2 * p.tt <= pass_threads(p.el, esz) ? 2 : 1;
+}
+
+ColConfig col_config(const Geom& g, const FftPlan& p, const ColDesc& d, int W, int esz) {
+  ColConfig c{};
+  c.w = W;
+  c.pitch = (p.buf + 15) / 16 * 16 + (W > 1 ? (esz == 4 ? 16 : 8) / W : 0);
+  const int most = d.nfwd > d.nder ? d.nfwd : d.nder;
+  auto bytes = [&](int f, int nbuf) {
+    return ((size_t)f * W * nbuf * c.pitch + 2 * (size_t)W * g.Ny) * 2 * esz;
+  };
+  const int target = esz == 4 ? 256 : 192;
+  int f = target / (p.tt * W);
+  if (f < 1) f = 1;
+  if (f > most) f = most > 0 ? most : 1;
+  const int rounds = most > 0 ? (most + f - 1) / f : 1;
+  f = most > 0 ? (most + rounds - 1) / rounds : 1;
+  while (f > 1 && bytes(f, 2) > kSmemCap / 2) --f;
+  c.fields = f;
+  c.one_buf = bytes(f, 2) > kSmemCap;
+  c.smem = bytes(f, c.one_buf ? 1 : 2);
+  c.threads = (f * W * p.tt + 31) / 32 * 32;
+  c.warp = p.tt * W <= 32 && 32 % (p.tt * W) == 0;
+  return c;
+}
+
+}  // namespace qg

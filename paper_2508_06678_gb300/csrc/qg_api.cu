@@ -73,30 +73,6 @@ bool valid_n(int n) {
   return m == 1;
 }
 
-FftPlan make_plan(int n) {
-  FftPlan p{};
-  p.n = n;
-  int m = n;
-  while (m % 8 == 0) { p.radix[p.npass++] = 8; m /= 8; }
-  if (m % 4 == 0) { p.radix[p.npass++] = 4; m /= 4; }
-  if (m % 2 == 0) { p.radix[p.npass++] = 2; m /= 2; }
-  while (m % 3 == 0) { p.radix[p.npass++] = 3; m /= 3; }
-  return p;
-}
-
-int max_items(int R) { return R == 3 ? 2 : 8 / R; }
-
-int threads_for(const FftPlan& p, int B, int floor_threads) {
-  int need = floor_threads;
-  for (int s = 0; s < p.npass; ++s) {
-    const int R = p.radix[s];
-    const int items = (p.n / R) * B;
-    const int t = (items + max_items(R) - 1) / max_items(R);
-    if (t > need) need = t;
-  }
-  return (need + 31) / 32 * 32;
-}
-
 // cos and sin of 2 pi j / n with the argument reduced exactly to [0, pi/4].
 void cos_sin_frac(long j, long n, double* c, double* s) {
   j %= n;
@@ -125,57 +101,6 @@ void cos_sin_frac(long j, long n, double* c, double* s) {
 }  // namespace
 
 namespace qg {
-// Non-first passes of the specialised FFT in order (radix-16 passes, then the
-// last pass of radix 2^(log2 n mod 4)); each contributes (R - 1) * NS entries
-// [r - 1][k] = W_n^(r k n / (NS R)).
-// The twiddled passes (every pass after the first) of the specialised engines, in order:
-// N = 2^p: radix 16 while possible, then one radix-8/4/2 pass; N = 3 * 2^p: radix 4 after the first
-// (radix-12) pass while a factor 4 remains, then one radix-2 pass for odd p.
-static void for_each_pass(int n, void (*fn)(int, int, int, void*), void* ctx) {
-  int off = 0;
-  if (n % 3 == 0) {
-    int m = n / 12, ns = 12;
-    for (; m >= 4; m /= 4, ns *= 4) {
-      fn(4, ns, off, ctx);
-      off += 3 * ns;
-    }
-    if (m == 2) fn(2, ns, off, ctx);
-    return;
-  }
-  int lg = 0;
-  while ((1 << lg) < n) ++lg;
-  const int np16 = lg / 4, rlast = 1 << (lg % 4);
-  int ns = 16;
-  for (int p = 1; p < np16; ++p, ns *= 16) {
-    fn(16, ns, off, ctx);
-    off += 15 * ns;
-  }
-  if (rlast > 1) fn(rlast, n / rlast, off, ctx);
-}
-
-int fast_pass_table_size(int n) {
-  int total = 0;
-  for_each_pass(n, [](int R, int NS, int off, void* c) { *(int*)c = off + (R - 1) * NS; }, &total);
-  return total;
-}
-
-void fast_pass_table(int n, const double* tw, double* out) {
-  struct Ctx { int n; const double* tw; double* out; } cx{n, tw, out};
-  for_each_pass(
-      n,
-      [](int R, int NS, int off, void* c) {
-        Ctx& x = *(Ctx*)c;
-        for (int r = 1; r < R; ++r)
-          for (int k = 0; k < NS; ++k) {
-            const long j = ((long)r * k * (x.n / (NS * R))) % x.n;
-            const size_t e = (size_t)off + (size_t)(r - 1) * NS + k;
-            x.out[2 * e] = x.tw[2 * j];
-            x.out[2 * e + 1] = x.tw[2 * j + 1];
-          }
-      },
-      &cx);
-}
-
 // Lets other translation units of the library report through qg_last_error().
 void set_last_error(const char* msg) { g_err = msg; }
 }  // namespace qg
@@ -189,10 +114,12 @@ struct qg_handle {
   qg_params par{};
   cudaStream_t stream = nullptr;
   FftPlan plan{};
-  int W = 4, col_threads = 256, row_threads = 256;
-  size_t col_smem = 0, row_smem = 0;
+  int W = 2;  // k_x columns per CTA of the column pass
   int ncolblk = 0;
-  bool fast = false;  // power-of-two grid served by the register-resident FFT kernels
+  // the passes that serve the grid: run-time transforms (FP64, and the smallest FP32 grids), or passes specialised
+  // for N that run a row's or column's transforms side by side (wide), or one after another with TMA tiles (fast)
+  bool wide = false, fast = false;
+  bool adj_fused = false;  // the adjoint's fused row passes fit in shared memory
   bool dynamic = false;
   double static_coeff = 0.0;
   int test_m2max = 0;  // largest |m|^2 the test filter keeps
@@ -231,8 +158,7 @@ struct qg_handle {
   cudaEvent_t adj_join_ev[8] = {};
   int adj_njoin = 0;
   int32_t adj_graph_launches[QG_NUM_KCLASS] = {};
-  void* tw = nullptr;
-  void* ptw = nullptr;  // per-pass twiddle table of the power-of-two kernels
+  void* ptw = nullptr;  // per-pass twiddle table of the handle's FFT engine
   void* visc_x = nullptr;
   void* visc_y = nullptr;
   void* phys = nullptr;
@@ -381,48 +307,44 @@ struct Bracket {
   }
 };
 
-template <typename T>
-cudaError_t row_fast_dispatch(qg_handle* h, const RowDesc& d) {
-  switch (h->g.n) {
-    case 256: return launch_row_fast<T, 256>(h->g, d, h->ptw, h->stream);
-    case 512: return launch_row_fast<T, 512>(h->g, d, h->ptw, h->stream);
-    case 1024: return launch_row_fast<T, 1024>(h->g, d, h->ptw, h->stream);
-    case 2048: return launch_row_fast<T, 2048>(h->g, d, h->ptw, h->stream);
-    case 4096: return launch_row_fast<T, 4096>(h->g, d, h->ptw, h->stream);
-    case 384: return launch_row_fast<T, 384>(h->g, d, h->ptw, h->stream);
-    case 768: return launch_row_fast<T, 768>(h->g, d, h->ptw, h->stream);
-    case 1536: return launch_row_fast<T, 1536>(h->g, d, h->ptw, h->stream);
-    case 3072: return launch_row_fast<T, 3072>(h->g, d, h->ptw, h->stream);
-    default: return cudaErrorInvalidValue;
-  }
+cudaError_t row_dispatch(qg_handle* h, const RowDesc& d) {
+  if (!h->fp32) return launch_row<double>(h->g, h->plan, d, h->ptw, h->stream);
+#define X(N) \
+  case N: return launch_row_fast<float, N>(h->g, d, h->ptw, h->stream);
+  if (h->fast) switch (h->g.n) { QG_FAST_GRIDS(X) default: return cudaErrorInvalidValue; }
+#undef X
+#define X(N) \
+  case N: return launch_row_wide<N>(h->g, h->plan, d, h->ptw, h->stream);
+  if (h->wide) switch (h->g.n) { QG_WIDE_GRIDS(X) default: return cudaErrorInvalidValue; }
+#undef X
+  return launch_row<float>(h->g, h->plan, d, h->ptw, h->stream);
 }
 
-template <typename T>
-cudaError_t col_fast_dispatch(qg_handle* h, const ColDesc& d) {
-  TmaSet tm;
-  memset(&tm, 0, sizeof(tm));
-  for (int f = 0; f < d.nfwd; ++f) {
-    const CUtensorMap* m = find_map(h, d.fin[f]);
-    if (!m) return cudaErrorInvalidValue;
-    tm.in[f] = *m;
+cudaError_t col_dispatch(qg_handle* h, const ColDesc& d) {
+  if (!h->fp32) return launch_col<double>(h->g, h->plan, d, h->ptw, h->W, h->stream);
+  if (h->fast) {
+    TmaSet tm;
+    memset(&tm, 0, sizeof(tm));
+    for (int f = 0; f < d.nfwd; ++f) {
+      const CUtensorMap* m = find_map(h, d.fin[f]);
+      if (!m) return cudaErrorInvalidValue;
+      tm.in[f] = *m;
+    }
+    for (int q = 0; q < d.nder; ++q) {
+      const CUtensorMap* m = find_map(h, d.dout[q]);
+      if (!m) return cudaErrorInvalidValue;
+      tm.out[q] = *m;
+    }
+#define X(N) \
+  case N: return launch_col_fast<float, N>(h->g, d, h->ptw, tm, h->stream);
+    switch (h->g.n) { QG_FAST_GRIDS(X) default: return cudaErrorInvalidValue; }
+#undef X
   }
-  for (int q = 0; q < d.nder; ++q) {
-    const CUtensorMap* m = find_map(h, d.dout[q]);
-    if (!m) return cudaErrorInvalidValue;
-    tm.out[q] = *m;
-  }
-  switch (h->g.n) {
-    case 256: return launch_col_fast<T, 256>(h->g, d, h->ptw, tm, h->stream);
-    case 512: return launch_col_fast<T, 512>(h->g, d, h->ptw, tm, h->stream);
-    case 1024: return launch_col_fast<T, 1024>(h->g, d, h->ptw, tm, h->stream);
-    case 2048: return launch_col_fast<T, 2048>(h->g, d, h->ptw, tm, h->stream);
-    case 4096: return launch_col_fast<T, 4096>(h->g, d, h->ptw, tm, h->stream);
-    case 384: return launch_col_fast<T, 384>(h->g, d, h->ptw, tm, h->stream);
-    case 768: return launch_col_fast<T, 768>(h->g, d, h->ptw, tm, h->stream);
-    case 1536: return launch_col_fast<T, 1536>(h->g, d, h->ptw, tm, h->stream);
-    case 3072: return launch_col_fast<T, 3072>(h->g, d, h->ptw, tm, h->stream);
-    default: return cudaErrorInvalidValue;
-  }
+#define X(N) \
+  case N: return launch_col_wide<N>(h->g, h->plan, d, h->ptw, h->W, h->stream);
+  if (h->wide) switch (h->g.n) { QG_WIDE_GRIDS(X) default: return cudaErrorInvalidValue; }
+#undef X
+  return launch_col<float>(h->g, h->plan, d, h->ptw, h->W, h->stream);
 }
 
 int run_row(qg_handle* h, RowDesc& d, int cls, bool use_flag = true) {
@@ -430,12 +352,7 @@ int run_row(qg_handle* h, RowDesc& d, int cls, bool use_flag = true) {
   d.err = h->flag;
   if (h->step_pdl) d.pdl = 1;
   Bracket br(h, cls);
-  cudaError_t e;
-  if (h->fast)
-    e = h->fp32 ? row_fast_dispatch<float>(h, d) : row_fast_dispatch<double>(h, d);
-  else
-    e = h->fp32 ? launch_row<float>(h->g, h->plan, d, h->tw, h->row_threads, h->row_smem, h->stream)
-                : launch_row<double>(h->g, h->plan, d, h->tw, h->row_threads, h->row_smem, h->stream);
+  const cudaError_t e = row_dispatch(h, d);
   br.done();
   if (e != cudaSuccess) return cuda_fail(e, "row pass launch");
   return QG_OK;
@@ -447,12 +364,7 @@ int run_col(qg_handle* h, ColDesc& d, int cls, bool use_flag = true) {
   if (h->step_pdl) d.pdl = 1;
   d.lean = h->lean_reduce;
   Bracket br(h, cls);
-  cudaError_t e;
-  if (h->fast)
-    e = h->fp32 ? col_fast_dispatch<float>(h, d) : col_fast_dispatch<double>(h, d);
-  else
-    e = h->fp32 ? launch_col<float>(h->g, h->plan, d, h->tw, h->W, h->col_threads, h->col_smem, h->stream)
-                : launch_col<double>(h->g, h->plan, d, h->tw, h->W, h->col_threads, h->col_smem, h->stream);
+  const cudaError_t e = col_dispatch(h, d);
   br.done();
   if (e != cudaSuccess) return cuda_fail(e, "column pass launch");
   return QG_OK;
@@ -535,7 +447,7 @@ int enqueue_step(qg_handle* h) {
     r.nout = h->nout;
     r.dx_mask = h->dx_mask;
     r.check_finite = 1;
-    for (int i = 0; i < h->nin; ++i) r.in[i] = h->X[i];
+    for (int i = 0; i < h->nder; ++i) r.in[i] = h->X[i];
     for (int i = 0; i < h->nout; ++i) r.out[i] = h->Y[i];
     if ((rc = run_row(h, r, QG_K_ROW_STAGE))) return rc;
 
@@ -666,7 +578,7 @@ int enqueue_step_ab2(qg_handle* h) {
   r.nout = h->nout;
   r.dx_mask = h->dx_mask;
   r.check_finite = 1;
-  for (int i = 0; i < h->nin; ++i) r.in[i] = h->X[i];
+  for (int i = 0; i < h->nder; ++i) r.in[i] = h->X[i];
   for (int i = 0; i < h->nout; ++i) r.out[i] = h->Y[i];
   if ((rc = run_row(h, r, QG_K_ROW_STAGE))) return rc;
   if (h->fac_b) {  // chi (u_total, v): X[0], X[1] hold the stage's u_total and v
@@ -853,7 +765,7 @@ int adj_to_spec_many(qg_handle* h, std::initializer_list<const void*> P, std::in
   const int n = (int)p.size();
   if (n < 1 || n > kAdjNM || (int)s.size() != n) return fail(QG_ERR_ARG, "adjoint: bad transform batch");
   int rc = QG_OK;
-  if (h->fast && n > 2) {
+  if (h->adj_fused && n > 2) {
     RowDesc r{};
     r.pdl = 1;  // the adjoint's chains of small launches overlap their launch latency
     r.prog = RP_COPY;
@@ -912,7 +824,7 @@ int adj_to_phys(qg_handle* h, const void* S, std::initializer_list<int> codes, s
   }
   int rc = run_col(h, c, QG_K_ADJ_COL, false);
   std::vector<void*> dst(P);
-  if (!rc && h->fast && dst.size() > 2) {
+  if (!rc && h->adj_fused && dst.size() > 2) {
     // every pair in one launch of the register-resident row pass
     RowDesc r{};
     r.pdl = 1;
@@ -1149,7 +1061,7 @@ int adj_forward_germano(qg_handle* h, int kind, const void* Sw, const void* SJ, 
   const double rp = std::pow(h->cl.test_ratio, kind == AK_SMAG ? 2 : 3);
   const double n4 = std::pow(double(h->g.n), 4);
   int rc = adj_combine(h, Swt, false, false, {{Sw, AM_ONE | AM_TESTF, 1.0}});
-  if (h->fast) {
+  if (h->adj_fused) {
     if (!rc) rc = adj_fused_fwd(h, kind, Swt, f0, T0, T1, T2);
   } else {
     if (!rc) rc = adj_stage_fields(h, Swt, kind, f0);
@@ -1180,7 +1092,7 @@ int adj_forward_stage(qg_handle* h, int kind, bool dyn, double C, const void* S0
   void* Sgx = S[kAdjStageS + 2 * s];
   void* Sgy = S[kAdjStageS + 2 * s + 1];
   int rc = QG_OK;
-  if (h->fast) {
+  if (h->adj_fused) {
     rc = adj_fused_fwd(h, kind, Sw, f0, S[8], Sgx, Sgy);
   } else {
     rc = adj_stage_fields(h, Sw, kind, f0);
@@ -1215,7 +1127,7 @@ int adj_reverse_germano(qg_handle* h, int kind, void* Slam_out, int s) {
   const int mu = kAdjDynMuP;
   int rc = adj_combine(h, Snu, false, false, {{SH, AM_ONE, 1.0}, {SM, AM_ONE, -2.0, C}});
   // outer group, at the test-level state, filtered afterwards: mu = M, derivatives of nu
-  if (h->fast) {
+  if (h->adj_fused) {
     if (!rc) rc = adj_derive(h, SM, {D_W}, 0);
     if (!rc) rc = adj_derive(h, Snu, {D_WX, D_WY}, 1);
   } else {
@@ -1227,20 +1139,20 @@ int adj_reverse_germano(qg_handle* h, int kind, void* Slam_out, int s) {
     if (pass == 1) {
       // inner group, at the stage state: mu = G M, derivatives of G nu
       rc = adj_combine(h, Sg, false, false, {{SM, AM_ONE | AM_TESTF, 1.0}});
-      if (h->fast) {
+      if (h->adj_fused) {
         if (!rc) rc = adj_derive(h, Sg, {D_W}, 0);
       } else {
         if (!rc) rc = adj_to_phys(h, Sg, {D_W}, {P[mu]});
       }
       if (!rc) rc = adj_combine(h, Sg, false, false, {{Snu, AM_ONE | AM_TESTF, 1.0}});
-      if (h->fast) {
+      if (h->adj_fused) {
         if (!rc) rc = adj_derive(h, Sg, {D_WX, D_WY}, 1);
       } else {
         if (!rc) rc = adj_to_phys(h, Sg, {D_WX, D_WY}, {P[7], P[8]});
         if (!rc) rc = adj_products(h, adj_prod_desc(h, kind, AP_ADJOINT, kAdjStageP + 6 * s, mu));
       }
     }
-    if (!rc && h->fast)
+    if (!rc && h->adj_fused)
       rc = adj_fused_rev_tail(h, kind, pass == 0 ? kAdjDynP + 6 * s : kAdjStageP + 6 * s);
     else if (!rc && kind == AK_SMAG)
       rc = adj_to_spec_many(h, {P[9], P[10], P[11], P[12], P[13], P[14], P[15], P[16]},
@@ -1311,14 +1223,14 @@ int adj_reverse_stage(qg_handle* h, int kind, bool dyn, double C, const void* Sl
     if (rc) return rc;
     if (urc) return urc;
   }
-  if (h->fast) {
+  if (h->adj_fused) {
     rc = adj_derive(h, Slam, {D_W, D_WX, D_WY}, 0);
     if (!rc) rc = adj_fused_rev_tail(h, kind, f0);
   } else {
     rc = adj_to_phys(h, Slam, {D_W, D_WX, D_WY}, {P[6], P[7], P[8]});
     if (!rc) rc = adj_products(h, adj_prod_desc(h, kind, AP_ADJOINT, f0));
   }
-  if (!rc && h->fast) {
+  if (!rc && h->adj_fused) {
     // the fused passes wrote S[8..]
   } else if (!rc && kind == AK_SMAG)
     rc = adj_to_spec_many(h, {P[9], P[10], P[11], P[12], P[13], P[14], P[15], P[16]},
@@ -1390,7 +1302,7 @@ int adj_step(qg_handle* h) {
     rc = adj_forward_stage(h, kind, dyn, C, S[0], S[s], S[s + 1], A[s], B[s], s);
   if (!rc) rc = adj_combine(h, S[3], false, false, {{S[3], AM_VISC, 1.0}});
   if (rc) return rc;
-  if (h->fac_b && h->fast) {
+  if (h->fac_b && h->adj_fused) {
     // the forward step's own Brinkman passes: (u_total, v) derived, scaled by the exact factor in one row pass,
     // curl taken in the column pass that transforms them
     rc = adj_derive(h, S[3], {D_U, D_V}, 0);
@@ -1458,7 +1370,7 @@ int adj_step(qg_handle* h) {
     }
     rc = adj_to_spec(h, P[2], lam, false);
   }
-  if (!rc && h->fac_b && h->fast) {
+  if (!rc && h->fac_b && h->adj_fused) {
     // w5 = T (d_x (f v) - d_y (f u)): lam <- -conj(dv) F[f lam_x] + conj(du) F[f lam_y], the scaling in one row pass
     rc = adj_derive(h, lam, {D_WX, D_WY}, 0);
     if (!rc) rc = adj_brinkman_row(h);
@@ -1866,7 +1778,6 @@ int qg_create(const qg_grid* grid, double beta, double U, const double* mask, co
   g.Ny = 2 * g.K + 1;
   g.SP = (g.Ny + 3) / 4 * 4;
   g.kscale = 2.0 * M_PI / grid->L;
-  h->plan = make_plan(n);
 
   int dev = 0, smem_optin = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -1887,7 +1798,7 @@ int qg_create(const qg_grid* grid, double beta, double U, const double* mask, co
     case QG_LEITH: h->row_prog = RP_LEITH; h->nout = 3; h->dx_mask = 0x2; break;
     case QG_SMAG:
       h->row_prog = RP_SMAG; h->nout = 3; h->dx_mask = 0x2;
-      h->der[nd++] = D_PXY; h->der[nd++] = D_PD;
+      h->der[2] = D_W;
       break;
     case QG_DLEITH:
       h->row_prog = RP_DLEITH; h->nout = 6; h->dx_mask = 0x12;
@@ -1895,63 +1806,32 @@ int qg_create(const qg_grid* grid, double beta, double U, const double* mask, co
       break;
     case QG_DSMAG:
       h->row_prog = RP_DSMAG; h->nout = 6; h->dx_mask = 0x12;
-      h->der[nd++] = D_PXY; h->der[nd++] = D_PD;
-      for (int i = 0; i < 4; ++i) h->der[nd++] = base4[i] | D_TEST;
-      h->der[nd++] = D_PXY | D_TEST; h->der[nd++] = D_PD | D_TEST;
+      h->der[2] = D_W;
+      for (int i = 0; i < 4; ++i) h->der[nd++] = h->der[i] | D_TEST;
       break;
   }
   h->nder = nd;
-  h->nin = nd;
+  // physical fields of a stage's row: the Smagorinsky programs form their strain pair from the stored four
+  h->nin = closure->kind == QG_SMAG ? 6 : closure->kind == QG_DSMAG ? 12 : nd;
 
-  // column tile width: 32-byte row segments, enough threads, shared memory fits
-  int W = h->fp32 ? 4 : 2;
-  const int col_max_threads = h->fp32 ? 1024 : 512;  // the kernels' launch bounds
-  for (;; W /= 2) {
-    const size_t sm = (size_t)n * W * csz + 2 * (size_t)W * g.Ny * csz;
-    const int th = threads_for(h->plan, W, 128);
-    if ((sm <= smem_cap && th <= col_max_threads) || W == 1) {
-      h->W = W;
-      h->col_smem = sm;
-      h->col_threads = th;
-      break;
-    }
-  }
-  if (h->col_smem > smem_cap || h->col_threads > col_max_threads) {
-    delete h;
-    return fail(QG_ERR_UNSUPPORTED, "qg_create: column pass does not fit (n=%d)", n);
-  }
+  // the row pass keeps a row's physical fields and one transform in shared memory
   const int nslot = h->nin > 2 ? h->nin : 2;
-  h->row_smem = (size_t)n * csz + (size_t)nslot * n * h->esz;
-  h->row_threads = threads_for(h->plan, 1, 256);
-  if (h->row_smem > smem_cap || h->row_threads > 512) {
+  const size_t row_smem = (size_t)n * csz + (size_t)nslot * n * h->esz;
+  if (row_smem > smem_cap) {
     delete h;
     return fail(QG_ERR_UNSUPPORTED, "qg_create: row pass needs %zu B of shared memory (n=%d, closure %d)",
-                h->row_smem, n, closure->kind);
+                row_smem, n, closure->kind);
   }
-  // 2^p and 3 * 2^p grids use the register-resident kernels (two k_x columns per CTA)
+  // the passes that serve this grid
   {
-    const bool spec = fast::fast_size(n);
-    int fw = 2;
-    switch (n) {
-      case 256: fw = fast_col_width<256>(); break;
-      case 512: fw = fast_col_width<512>(); break;
-      case 1024: fw = fast_col_width<1024>(); break;
-      case 2048: fw = fast_col_width<2048>(); break;
-      case 4096: fw = fast_col_width<4096>(); break;
-      case 384: fw = fast_col_width<384>(); break;
-      case 768: fw = fast_col_width<768>(); break;
-      case 1536: fw = fast_col_width<1536>(); break;
-      case 3072: fw = fast_col_width<3072>(); break;
-    }
-    const size_t dense = (size_t)n * fw * csz, padded = (size_t)fw * (n + n / 16 + 16 / fw) * csz;
-    const size_t fast_col_smem = 3 * (((dense > padded ? dense : padded) + 1023) / 1024 * 1024) + 1024;
-    const int tt = spec ? n / fast::elems_per_thread(n) : 1;
-    const int rows = tt >= QG_ROW_CTA_THREADS ? 1 : QG_ROW_CTA_THREADS / tt;  // rows per CTA of the row pass
-    const size_t fast_row_smem = (size_t)2 * rows * (n + n / 16) * csz;
-    h->fast = spec && fast_col_smem <= smem_cap && fast_row_smem <= smem_cap;
-    if (getenv("QG_FORCE_GENERIC")) h->fast = false;
-    if (const char* inj = getenv("QG_INJECT_TMA_STALL")) h->inject_stall = h->fast ? atoi(inj) + 1 : 0;
-    if (h->fast) h->W = fw;
+    const bool generic = getenv("QG_FORCE_GENERIC") != nullptr;
+    h->fast = h->fp32 && !generic && fast_grid(n);
+    h->wide = h->fp32 && !generic && wide_grid(n);
+    h->plan = fft_plan(n, h->fast || h->wide ? fft_elems(n, 4) : rt_elems(n, (int)h->esz));
+    if (const char* inj = getenv("QG_INJECT_TMA_STALL")) h->inject_stall = atoi(inj) + 1;
+    h->W = h->fast ? kFastWidth : col_width(h->plan, (int)h->esz);
+    const size_t adj_slots = closure->kind == QG_NONE ? 4 : closure->kind == QG_LEITH || closure->kind == QG_DLEITH ? 6 : 8;
+    h->adj_fused = h->fast || adj_slots * n * h->esz + h->plan.buf * csz <= smem_cap;
   }
   g.Kcp = (g.Kc + h->W - 1) / h->W * h->W;
   g.IP = g.Kcp;
@@ -1967,7 +1847,7 @@ int qg_create(const qg_grid* grid, double beta, double U, const double* mask, co
   if (!rc && h->dynamic) rc = dalloc(h, &h->jh, spec_bytes);
   if (!rc && h->dynamic) rc = dalloc(h, &h->dh, spec_bytes);
   for (int i = 0; i < 3 && !rc && h->dynamic && h->fast && h->fp32; ++i) rc = dalloc(h, &h->red_scr[i], spec_bytes);
-  for (int i = 0; i < h->nin && !rc; ++i) rc = dalloc(h, &h->X[i], mixed_bytes);
+  for (int i = 0; i < h->nder && !rc; ++i) rc = dalloc(h, &h->X[i], mixed_bytes);
   const int ny = h->nout > 2 ? h->nout : 2;
   for (int i = 0; i < ny && !rc; ++i) rc = dalloc(h, &h->Y[i], mixed_bytes);
   if (h->scheme == QG_SCHEME_AB2CN) {
@@ -1978,7 +1858,6 @@ int qg_create(const qg_grid* grid, double beta, double U, const double* mask, co
     if (!rc && mask && h->dynamic) rc = dalloc(h, &h->bh, spec_bytes);
   }
   if (!rc) rc = dalloc(h, &h->phys, phys_bytes);
-  if (!rc) rc = dalloc(h, &h->tw, (size_t)n * csz);
   if (!rc) rc = dalloc(h, &h->visc_x, (size_t)g.Kcp * h->esz);
   if (!rc) rc = dalloc(h, &h->visc_y, (size_t)g.SP * h->esz);
   if (!rc) rc = dalloc(h, (void**)&h->partials, (size_t)2 * h->ncolblk * sizeof(double));
@@ -2008,16 +1887,23 @@ int qg_create(const qg_grid* grid, double beta, double U, const double* mask, co
       tw[2 * j] = c;
       tw[2 * j + 1] = -s;
     }
-    if ((rc = upload_real(h, h->tw, tw))) { delete h; return rc; }
-    if (h->fast) {
-      const int nt = fast_pass_table_size(n);
-      std::vector<double> pt(2 * (size_t)(nt > 0 ? nt : 1), 0.0);
-      fast_pass_table(n, tw.data(), pt.data());
-      if ((rc = dalloc(h, &h->ptw, pt.size() / 2 * csz)) || (rc = upload_real(h, h->ptw, pt))) {
-        delete h;
-        return rc;
-      }
+    std::vector<double> pt(2 * (size_t)h->plan.table);
+    for (int e = 0; e < h->plan.table; ++e) {
+      const int j = fft_table_exponent(h->plan, e);
+      pt[2 * e] = tw[2 * j];
+      pt[2 * e + 1] = tw[2 * j + 1];
     }
+    if ((rc = dalloc(h, &h->ptw, pt.size() / 2 * csz)) || (rc = upload_real(h, h->ptw, pt))) {
+      delete h;
+      return rc;
+    }
+  }
+  if (!h->fp32) {
+    std::vector<double> kt(n / 2 + 1);
+    for (int m = 0; m <= n / 2; ++m) kt[m] = g.kscale * m;
+    void* p = nullptr;
+    if ((rc = dalloc(h, &p, kt.size() * 8)) || (rc = upload_real(h, p, kt))) { delete h; return rc; }
+    g.kt = static_cast<const double*>(p);
   }
   // tensor maps of every mixed array for the TMA column pass
   if (h->fast) {

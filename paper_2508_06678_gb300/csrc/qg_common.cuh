@@ -67,7 +67,22 @@ struct Geom {
   int SP;     // spectral column pitch (complex elements)
   int IP;     // mixed-array row pitch (complex elements) = Kcp
   double kscale;  // 2 pi / L
+  const double* kt;  // FP64 handles: kscale * m for m = 0 .. N / 2 (a conversion from int costs an FP64 operation)
 };
+
+// wavenumber 2 pi m / L in the working precision
+template <typename T> __device__ __forceinline__ T wavenumber(const Geom& g, int m);
+template <> __device__ __forceinline__ float wavenumber<float>(const Geom& g, int m) { return float(g.kscale) * float(m); }
+template <> __device__ __forceinline__ double wavenumber<double>(const Geom& g, int m) {
+  const double k = __ldg(g.kt + (m < 0 ? -m : m));
+  return m < 0 ? -k : k;
+}
+
+// infinite or NaN, by the exponent bits (an FP64 comparison costs an FP64 operation)
+__device__ __forceinline__ bool nonfinite(float v) { return (__float_as_uint(v) & 0x7f800000u) == 0x7f800000u; }
+__device__ __forceinline__ bool nonfinite(double v) {
+  return ((unsigned)__double2hiint(v) & 0x7ff00000u) == 0x7ff00000u;
+}
 
 __host__ __device__ __forceinline__ int my_of_r(const Geom& g, int r) { return r <= g.K ? r : r - g.Ny; }
 // row of an N-point k_y sequence (FFT order) holding spectral index r
@@ -97,7 +112,7 @@ enum DerCode : int {
 enum RowProg : int {
   RP_NONE = 0,    // (u, v, wx, wy) -> J
   RP_LEITH = 1,   // (u, v, wx, wy) -> J, g wx, g wy with g = |grad w|
-  RP_SMAG = 2,    // (u, v, wx, wy, pxy, pd) -> J, g wx, g wy with g = |S|
+  RP_SMAG = 2,    // (u, v, w, wy) -> J, g wx, g wy with g = |S| (wx and the strain pair formed from them on loading)
   RP_DLEITH = 3,  // RP_LEITH at grid and test level
   RP_DSMAG = 4,   // RP_SMAG at grid and test level
   RP_SCALE = 5,   // f_i * factor(x, y) for each input (Brinkman, sponge)

@@ -5,13 +5,43 @@
 
 namespace qg {
 
+// Launch shape of the row pass: rows per CTA, groups (transforms side by side), physical rows kept in shared memory
+// per row (slots).
+struct RowConfig {
+  int rows, groups, threads, nslot, one_buf, warp;
+  size_t smem;
+};
+RowConfig row_config(const FftPlan& p, const RowDesc& d, int esz);
 template <typename T>
-cudaError_t launch_row(const Geom& g, const FftPlan& plan, const RowDesc& d, const void* tw, int threads,
-                       size_t smem, cudaStream_t st);
+cudaError_t launch_row(const Geom& g, const FftPlan& plan, const RowDesc& d, const void* tw, cudaStream_t st);
 
+// Launch shape of the column pass: w columns per CTA, fields transformed side by side, buffer pitch.
+struct ColConfig {
+  int w, fields, threads, pitch, one_buf, warp;
+  size_t smem;
+};
+ColConfig col_config(const Geom& g, const FftPlan& p, const ColDesc& d, int W, int esz);
 template <typename T>
-cudaError_t launch_col(const Geom& g, const FftPlan& plan, const ColDesc& d, const void* tw, int W, int threads,
-                       size_t smem, cudaStream_t st);
+cudaError_t launch_col(const Geom& g, const FftPlan& plan, const ColDesc& d, const void* tw, int W, cudaStream_t st);
+// columns per CTA of the column pass (the mixed arrays' pitch is a multiple of it)
+int col_width(const FftPlan& p, int esz);
+
+// FP32 grids with passes specialised for N (grid_<N>.cu): transforms side by side up to 324, one after another from
+// 384 on.  Measured around the line, us per step on an idle GPU: dynamic Smagorinsky 256^2 91 side by side and 143 one
+// after another, dynamic Leith 384^2 127 and 138, Smagorinsky 384^2 96 and 85, Leith 512^2 101 and 72.
+#define QG_WIDE_GRIDS(X) X(64) X(72) X(96) X(108) X(128) X(144) X(162) X(192) X(216) X(256) X(288) X(324)
+#define QG_FAST_GRIDS(X)                                                                         \
+  X(384) X(432) X(486) X(512) X(576) X(648) X(768) X(864) X(972) X(1024) X(1152) X(1296) \
+  X(1458) X(1536) X(1728) X(1944) X(2048) X(2304) X(2592) X(2916) X(3072) X(3456) X(3888) X(4096)
+#define X(N) || n == N
+constexpr bool wide_grid(int n) { return false QG_WIDE_GRIDS(X); }
+constexpr bool fast_grid(int n) { return false QG_FAST_GRIDS(X); }
+#undef X
+template <int N>
+cudaError_t launch_row_wide(const Geom& g, const FftPlan& plan, const RowDesc& d, const void* tw, cudaStream_t st);
+template <int N>
+cudaError_t launch_col_wide(const Geom& g, const FftPlan& plan, const ColDesc& d, const void* tw, int W,
+                            cudaStream_t st);
 
 // Spectral diagnostics: out[0] = sum w |k|^2 |psi|^2, out[1] = sum w |w|^2 over the stored half spectrum
 // (w = 1 on the k_x = 0 column, else 2), FP64, deterministic two-level reduction.

@@ -12,6 +12,9 @@
 namespace qg {
 namespace tma {
 
+// bounded device waits: about one second of SM clocks
+constexpr long long kWaitCycles = 2000000000LL;
+
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
