@@ -30,6 +30,8 @@ constexpr int kThreads = 256;
 
 }  // namespace
 
+// Bound by its FP64 operations (which the FP32 adjoint takes too): the wavenumbers, 1 / |k|^2 and the viscous factor
+// come from tables, and a term is a factor and two FMAs.
 template <typename T>
 __global__ void __launch_bounds__(kThreads) adj_combine_kernel(Geom g, AdjCombine a) {
   pdl_enter();
@@ -43,38 +45,41 @@ __global__ void __launch_bounds__(kThreads) adj_combine_kernel(Geom g, AdjCombin
       continue;
     }
     const int my = my_of_r(g, r);
-    const double kx = g.kscale * c, ky = g.kscale * my;
-    const double k2 = kx * kx + ky * ky;
-    const double ik2 = k2 > 0.0 ? 1.0 / k2 : 0.0;
+    const double kx = g.kt[c], ky = my < 0 ? -g.kt[-my] : g.kt[my];
+    const double ik2 = a.ik2[e];
+    const double kxi = kx * ik2, kyi = ky * ik2;
     double re = 0.0, im = 0.0;
     if (a.accumulate) {
       const C o = out[e];
       re = double(o.x);
       im = double(o.y);
     }
-    const bool in_test = (long)c * c + (long)my * my <= (long)a.test_m2max;
+    const bool in_test = c * c + my * my <= a.test_m2max;
     for (int j = 0; j < a.nterm; ++j) {
       const int code = a.term[j].code;
       if ((code & AM_TESTF) && !in_test) continue;
       const C x = ld<T>(a.term[j].in, e);
       const double xr = double(x.x), xi = double(x.y);
-      const double cf = a.term[j].cptr ? a.term[j].coef * a.term[j].cptr[0] : a.term[j].coef;
-      double mr = 0.0, mi = 0.0;  // multiplier m = mr + i mi
+      double f = a.term[j].coef;
+      if (a.term[j].cptr) f *= a.term[j].cptr[0];
+      bool imag = true;  // the multiplier is i f, else f
       switch (code & 0xff) {
-        case AM_ONE: mr = 1.0; break;
-        case AM_CU: mi = -ky * ik2; break;  // conj(i k_y / |k|^2): transpose of w -> u
-        case AM_CV: mi = kx * ik2; break;   // conj(-i k_x / |k|^2): transpose of w -> v
-        case AM_CX: mi = -kx; break;        // conj(i k_x)
-        case AM_CY: mi = -ky; break;        // conj(i k_y)
-        case AM_IX: mi = kx; break;
-        case AM_IY: mi = ky; break;
-        case AM_XY: mr = kx * ky * ik2; break;              // w -> psi_xy (real)
-        case AM_DD: mr = (kx * kx - ky * ky) * ik2; break;  // w -> psi_xx - psi_yy (real)
-        case AM_VISC: mr = exp(-(a.nu * k2 + a.mu) * a.dt); break;
-        default: break;
+        case AM_CU: f *= -kyi; break;  // conj(i k_y / |k|^2): transpose of w -> u
+        case AM_CV: f *= kxi; break;   // conj(-i k_x / |k|^2): transpose of w -> v
+        case AM_CX: f *= -kx; break;   // conj(i k_x)
+        case AM_CY: f *= -ky; break;   // conj(i k_y)
+        case AM_IX: f *= kx; break;
+        case AM_IY: f *= ky; break;
+        case AM_XY: f *= kx * kyi; imag = false; break;             // w -> psi_xy (real)
+        case AM_DD: f *= kx * kxi - ky * kyi; imag = false; break;  // w -> psi_xx - psi_yy (real)
+        case AM_VISC:
+          f *= a.visc_x ? a.visc_x[c] * a.visc_y[r] * a.visc_mu : exp(-(a.nu * (kx * kx + ky * ky) + a.mu) * a.dt);
+          imag = false;
+          break;
+        default: imag = false; break;  // AM_ONE
       }
-      re += cf * (mr * xr - mi * xi);
-      im += cf * (mr * xi + mi * xr);
+      re = fma(imag ? -f : f, imag ? xi : xr, re);
+      im = fma(f, imag ? xr : xi, im);
     }
     if (a.zero_mean && c == 0 && my == 0) re = im = 0.0;
     out[e] = mk<C>(T(re), T(im));
@@ -273,36 +278,36 @@ unsigned grid_for(size_t count) {
 
 template <typename T>
 cudaError_t launch_adj_combine(const Geom& g, const AdjCombine& a, cudaStream_t st) {
-  return launch_pdl(true, adj_combine_kernel<T>, dim3(grid_for((size_t)g.Kcp * g.SP)), dim3(kThreads), 0, st, g, a);
+  return launch_pdl(sizeof(T) == 4, adj_combine_kernel<T>, dim3(grid_for((size_t)g.Kcp * g.SP)), dim3(kThreads), 0, st, g, a);
 }
 
 template <typename T>
 cudaError_t launch_adj_products(size_t count, const AdjProducts& a, cudaStream_t st) {
-  return launch_pdl(true, adj_products_kernel<T>, dim3(grid_for(count)), dim3(kThreads), 0, st, count, a);
+  return launch_pdl(sizeof(T) == 4, adj_products_kernel<T>, dim3(grid_for(count)), dim3(kThreads), 0, st, count, a);
 }
 
 template <typename T>
 cudaError_t launch_adj_scale(size_t count, const void* f, const void* x0, double s0, void* out0, const void* x1,
                              double s1, void* out1, cudaStream_t st) {
-  return launch_pdl(true, adj_scale_kernel<T>, dim3(grid_for(count)), dim3(kThreads), 0, st, count, f, x0, T(s0), out0, x1,
+  return launch_pdl(sizeof(T) == 4, adj_scale_kernel<T>, dim3(grid_for(count)), dim3(kThreads), 0, st, count, f, x0, T(s0), out0, x1,
                     T(s1), out1);
 }
 
 template <typename T>
 cudaError_t launch_adj_spec_dot(const Geom& g, const void* A, const void* B, const AdjDotOut& o, cudaStream_t st) {
-  return launch_pdl(true, adj_spec_dot_kernel<T>, dim3(kAdjDotBlocks), dim3(kThreads), 0, st, g, A, B, o);
+  return launch_pdl(sizeof(T) == 4, adj_spec_dot_kernel<T>, dim3(kAdjDotBlocks), dim3(kThreads), 0, st, g, A, B, o);
 }
 
 template <typename T>
 cudaError_t launch_adj_germano_dots(const Geom& g, const void* H, const void* M, const AdjDotOut& o,
                                     cudaStream_t st) {
-  return launch_pdl(true, adj_germano_dots_kernel<T>, dim3(kAdjDotBlocks), dim3(kThreads), 0, st, g, H, M, o);
+  return launch_pdl(sizeof(T) == 4, adj_germano_dots_kernel<T>, dim3(kAdjDotBlocks), dim3(kThreads), 0, st, g, H, M, o);
 }
 
 template <typename T>
 cudaError_t launch_adj_phys_dot(size_t count, const void* X, const void* Y, const void* Z, const AdjDotOut& o,
                                 cudaStream_t st) {
-  return launch_pdl(true, adj_phys_dot_kernel<T>, dim3(kAdjDotBlocks), dim3(kThreads), 0, st, count, X, Y, Z, o);
+  return launch_pdl(sizeof(T) == 4, adj_phys_dot_kernel<T>, dim3(kAdjDotBlocks), dim3(kThreads), 0, st, count, X, Y, Z, o);
 }
 
 #define QG_ADJ_INST(T)                                                                                         \

@@ -53,6 +53,7 @@ void make_grid(Grid& G, int n, int K, double L, int nslot) {
   g.Ny = 2 * K + 1;
   g.SP = (g.Ny + 3) / 4 * 4;
   g.kscale = 2.0 * M_PI / L;
+  g.kscale_f = (float)g.kscale;
   G.plan = fft_plan(n, rt_elems(n, 8));
   G.W = col_width(G.plan, 8);
   g.Kcp = (g.Kc + G.W - 1) / G.W * G.W;

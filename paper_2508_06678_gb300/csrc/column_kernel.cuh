@@ -19,22 +19,10 @@
 
 #include "fft.cuh"
 #include "qg_kernels.h"
+#include "spectral.cuh"
 #include "tma.cuh"
 
 namespace qg {
-
-template <typename T> struct InvK2;
-template <> struct InvK2<double> {
-  __device__ static double get(double ks2, int m2) { return m2 == 0 ? 0.0 : 1.0 / (ks2 * double(m2)); }
-};
-template <> struct InvK2<float> {
-  // the few smallest wavenumbers are inverted in FP64 before rounding
-  __device__ static float get(double ks2, int m2) {
-    if (m2 == 0) return 0.f;
-    if (m2 <= 16) return float(1.0 / (ks2 * double(m2)));
-    return 1.f / (float(ks2) * float(m2));
-  }
-};
 
 // A CTA's groups of TT threads transform c.fields fields of its W columns side by side (thread = (field, position,
 // column), columns fastest so that a warp's accesses to a row of the mixed arrays are adjacent).  With one field at
@@ -44,8 +32,8 @@ template <> struct InvK2<float> {
 // (both over N^2) wait in shared memory for the derived fields, so 1 / |k|^2 is formed once per mode.
 template <typename T, class Sh, int OP>
 __global__ void __launch_bounds__(pass_threads(Sh::EL, sizeof(T))) col_kernel(Geom g, Sh sh, ColConfig cf, ColDesc d,
-                                                                 const cplx_t<T>* __restrict__ tw) {
-  pdl_enter();
+                                                                 const __grid_constant__ ColScalars<T> cs,
+                                                                 const cplx_t<T>* __restrict__ twg) {
   using C = cplx_t<T>;
   constexpr int EL = Sh::EL;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -55,21 +43,25 @@ __global__ void __launch_bounds__(pass_threads(Sh::EL, sizeof(T))) col_kernel(Ge
   const int tid = threadIdx.x, nt = blockDim.x;
   const int nbuf = cf.one_buf ? 1 : 2;
   const int cp = cf.pitch;  // complex elements of one exchange buffer
-  C* const bufs = reinterpret_cast<C*>(smem_raw);
+  C* const tws = reinterpret_cast<C*>(smem_raw);
+  C* const bufs = tws + (tw_shared(sh.table()) ? sh.table() : 0);
+  const C* tw = tw_stage(twg, sh.table(), tws);
+  pdl_enter();
+  const int stop = d.flag ? *reinterpret_cast<volatile int*>(d.flag) : 0;
   C* const slotA = bufs + (size_t)F * W * nbuf * cp;  // [W][Ny]
   C* const slotB = slotA + (size_t)W * Ny;            // [W][Ny]
-  const int c0 = blockIdx.x * W;
+  // this CTA's column tile and its part of the tile's outgoing fields
+  const int over = (int)blockIdx.x - cf.full;
+  const int tile = over < 0 ? blockIdx.x : cf.full + over / cf.split;
+  const int part = over < 0 ? 0 : over % cf.split, nparts = over < 0 ? 1 : cf.split;
+  const int c0 = tile * W;
   const int nspec = W * Ny;
-  const double ks2 = g.kscale * g.kscale;
   // extents for the bounds-checked debug build
   int* const st = d.err;
   const long long n_mixed = (long long)N * g.IP, n_spec = (long long)g.Kcp * g.SP;
   const long long n_part = 2LL * gridDim.x;  // Germano partial sums: two per column CTA
   (void)n_mixed; (void)n_spec; (void)n_part; (void)st;
 
-  if (d.flag) {
-    if (__syncthreads_or(*reinterpret_cast<volatile int*>(d.flag) != 0)) return;
-  }
 
   if (d.stall_cta1 == (int)blockIdx.x + 1 && d.nfwd > 0) {
     // injected stall (failure-handling test): a wait for a tile that is never requested runs out after its bound
@@ -102,8 +94,8 @@ __global__ void __launch_bounds__(pass_threads(Sh::EL, sizeof(T))) col_kernel(Ge
   C* ws = reinterpret_cast<C*>(d.ws);
   C* jh = reinterpret_cast<C*>(d.jh);
   C* dh = reinterpret_cast<C*>(d.dh);
-  const T rpow = T(d.rpow);
-  const T inv_eta = T(d.inv_eta);
+  const T rpow = cs.rpow;
+  const T inv_eta = cs.inv_eta;
   GermanoAcc<T> acc_hm, acc_mm;
 
   // mode r of column cc in the forward transform X of field f: what the op keeps of it
@@ -185,7 +177,7 @@ __global__ void __launch_bounds__(pass_threads(Sh::EL, sizeof(T))) col_kernel(Ge
   // arrays stay zero there
   int nder = 0;
   for (int q = 0; q < d.nder; ++q) {
-    if ((d.der[q] & D_TEST) && c0 > d.test_kmax) continue;
+    if (((d.der[q] & D_TEST) && c0 > d.test_kmax) || q % nparts != part) continue;
     if (tid == 0) dlist[nder] = q;
     ++nder;
   }
@@ -193,68 +185,32 @@ __global__ void __launch_bounds__(pass_threads(Sh::EL, sizeof(T))) col_kernel(Ge
 #pragma unroll 1
   for (int it = 0; it <= nfr + nir; ++it) {
     if (it == nfr) {
-      if (OP == CO_FORWARD_N) return;  // every field's band is stored
-      __syncthreads();                   // the slots (and dlist) are complete
-      if (OP == CO_DYN_REDUCE) {
-        // deterministic block reduction of the Germano partial sums
-        double hm = acc_hm.value(), mm = acc_mm.value();
-        for (int o = 16; o > 0; o >>= 1) {
-          hm += __shfl_down_sync(0xffffffffu, hm, o);
-          mm += __shfl_down_sync(0xffffffffu, mm, o);
-        }
-        const int lane = tid & 31, wid = tid >> 5;
-        if (lane == 0) {
-          red[0][wid] = hm;
-          red[1][wid] = mm;
-        }
-        __syncthreads();
-        if (wid == 0) {
-          const int nw = (nt + 31) >> 5;
-          hm = lane < nw ? red[0][lane] : 0.0;
-          mm = lane < nw ? red[1][lane] : 0.0;
-          for (int o = 16; o > 0; o >>= 1) {
-            hm += __shfl_down_sync(0xffffffffu, hm, o);
-            mm += __shfl_down_sync(0xffffffffu, mm, o);
-          }
-          if (lane == 0) {
-            QG_ST(d.partials, 2LL * blockIdx.x, n_part, st, hm);
-            QG_ST(d.partials, 2LL * blockIdx.x + 1, n_part, st, mm);
-          }
-        }
+      if constexpr (OP == CO_FORWARD_N) return;  // every field's band is stored
+      T coeff = cs.coeff;
+      if constexpr (OP == CO_DYN_COMBINE || OP == CO_AB2CN_COMBINE) {
+        if (!germano_coefficient(d.partials, d.npartials, red, nt, stop, d.coeff_out, st)) return;
+        coeff = T(red[0][0]);
+      } else if (__syncthreads_or(nfr == 0 ? stop : 0)) {  // also completes the slots and dlist
         return;
       }
-
-      // ---- coefficient of the dynamic closures from the partial sums (same order in every CTA)
-      T coeff = T(d.coeff);
-      if (OP == CO_DYN_COMBINE || OP == CO_AB2CN_COMBINE) {
-        if (tid < 32) {
-          double a = 0.0, b = 0.0;
-          for (int i = tid; i < d.npartials; i += 32) {
-            a += QG_LD(d.partials, 2LL * i, n_part, st);
-            b += QG_LD(d.partials, 2LL * i + 1, n_part, st);
-          }
-          for (int o = 16; o > 0; o >>= 1) {
-            a += __shfl_down_sync(0xffffffffu, a, o);
-            b += __shfl_down_sync(0xffffffffu, b, o);
-          }
-          if (tid == 0) {
-            const double Cc = b > 0.0 ? fmax(0.0, a / b) : 0.0;
-            red[0][0] = Cc;
-            if (blockIdx.x == 0 && d.coeff_out) *d.coeff_out = Cc;
-          }
+      if constexpr (OP == CO_DYN_REDUCE) {
+        // the CTA's Germano partial sums
+        pair_sum(acc_hm.value(), acc_mm.value(), red, (nt + 31) >> 5);
+        if (tid == 0) {
+          QG_ST(d.partials, 2LL * blockIdx.x, n_part, st, red[0][0]);
+          QG_ST(d.partials, 2LL * blockIdx.x + 1, n_part, st, red[1][0]);
         }
-        __syncthreads();
-        coeff = T(red[0][0]);
+        return;
       }
 
       // ---- new vorticity spectrum for the owned columns.  The modes go in batches whose global loads are all
       // issued before any of the batch's stores: the state arrays may alias as far as the compiler can tell, so a
       // load placed after a store would wait for that store's round trip.
-      const T dt = T(d.dt), a_rk = T(d.a), b_rk = T(d.b), beta = T(d.beta);
+      const T dt = cs.dt, a_rk = cs.a, b_rk = cs.b, beta = cs.beta;
       const T* vx = reinterpret_cast<const T*>(d.visc_x);
       const T* vy = reinterpret_cast<const T*>(d.visc_y);
-      const T vmu = T(d.visc_mu);
-      const T scale = T(1.0 / (double(N) * double(N)));
+      const T vmu = cs.visc_mu, scale = cs.scale;
+      const T* ik2t = reinterpret_cast<const T*>(d.ik2);
       const C* bhp = reinterpret_cast<const C*>(d.bh);
       C* ep = reinterpret_cast<C*>(d.eprev);
       C* wsp = reinterpret_cast<C*>(d.wss);
@@ -263,13 +219,14 @@ __global__ void __launch_bounds__(pass_threads(Sh::EL, sizeof(T))) col_kernel(Ge
         // per op: u0 = w^n (or w* in the AB2CN final), u1 = stage field or E_prev, u2 = J, u3 = D, u4 = Brinkman
         // forcing, u5 = previous w*; vf = viscous factor
         C u0[GB], u1[GB], u2[GB], u3[GB], u4[GB], u5[GB];
-        T vf[GB];
+        T vf[GB], ik[GB];
 #pragma unroll
         for (int q = 0; q < GB; ++q) {
           const int e = e0 + q * nt;
           const C z = mk<C>(T(0), T(0));
           u0[q] = z; u1[q] = z; u2[q] = z; u3[q] = z; u4[q] = z; u5[q] = z;
           vf[q] = T(1);
+          ik[q] = T(0);
           const int cc = e / Ny, r = e - cc * Ny, mx = c0 + cc;
           if (e < nspec && mx < g.Kc) {
             const int gi = mx * g.SP + r;
@@ -300,6 +257,9 @@ __global__ void __launch_bounds__(pass_threads(Sh::EL, sizeof(T))) col_kernel(Ge
               case CO_AB2CN_FINAL: u0[q] = QG_LD(wsp, gi, n_spec, st); break;
               default: break;
             }
+            // FP64: 1 / |k|^2 from the handle's table (a division is some ten FP64 operations a mode)
+            const int my = my_of_r(g, r);
+            ik[q] = sizeof(T) == 8 && ik2t ? QG_LD(ik2t, gi, n_spec, st) : inv_k2<T>(cs, mx * mx + my * my);
             if (d.viscous) vf[q] = QG_LD(vx, mx, g.Kcp, st) * QG_LD(vy, r, g.SP, st) * vmu;
           }
         }
@@ -312,7 +272,7 @@ __global__ void __launch_bounds__(pass_threads(Sh::EL, sizeof(T))) col_kernel(Ge
           const int m2 = mx * mx + my * my;
           const int gi = mx * g.SP + r;
           C wn = mk<C>(T(0), T(0));
-          const T ik2 = InvK2<T>::get(ks2, m2);
+          const T ik2 = ik[q];
           if (mx < g.Kc) {
             switch (OP) {
               case CO_DERIVE:
@@ -349,10 +309,10 @@ __global__ void __launch_bounds__(pass_threads(Sh::EL, sizeof(T))) col_kernel(Ge
                 }
                 const C Ep = d.ab2_first ? E : u1[q];
                 QG_ST(ep, gi, n_spec, st, E);
-                const T k2 = T(ks2) * T(m2);
+                const T k2 = cs.ks2 * T(m2);
                 const T kx = wavenumber<T>(g, mx);
                 const T hdt = T(0.5) * dt;
-                const T lre = -(T(d.nu) * k2 + T(d.mu));
+                const T lre = -(cs.nu * k2 + cs.mu);
                 const T lim = beta * kx * ik2;
                 const C wz = u0[q];
                 const C ab = mk<C>(T(1.5) * E.x - T(0.5) * Ep.x, T(1.5) * E.y - T(0.5) * Ep.y);
@@ -378,8 +338,8 @@ __global__ void __launch_bounds__(pass_threads(Sh::EL, sizeof(T))) col_kernel(Ge
             }
             if (d.viscous) wn = cscale(wn, vf[q]);
             if (d.zero_mean && m2 == 0) wn = mk<C>(T(0), T(0));
-            if (d.store_ws) QG_ST(reinterpret_cast<C*>(d.ws_out), gi, n_spec, st, wn);
-            if (d.store_w0) QG_ST(w0, gi, n_spec, st, wn);
+            if (d.store_ws && part == 0) QG_ST(reinterpret_cast<C*>(d.ws_out), gi, n_spec, st, wn);
+            if (d.store_w0 && part == 0) QG_ST(w0, gi, n_spec, st, wn);
             if (OP == CO_FORWARD2) {  // the second field, treated like the first
               C wb = QG_LD(slotB, e, nspec, st);
               if (d.viscous) wb = cscale(wb, vf[q]);
@@ -435,12 +395,14 @@ __global__ void __launch_bounds__(pass_threads(Sh::EL, sizeof(T))) col_kernel(Ge
               default: v = s; break;
             }
           }
-          if ((code & 7) == D_U && mx == 0 && my == 0) v = mk<C>(T(d.U), T(0));
+          if ((code & 7) == D_U && mx == 0 && my == 0) v = mk<C>(cs.U, T(0));
         }
         x[m] = mk<C>(v.y, v.x);
       }
     }
 
+    // the status flag's load has overlapped the inputs'; the barrier also completes the twiddle table
+    if (it == 0 && fwd && __syncthreads_or(stop)) return;
     sh.run(x, t, fb, tw);
 
     if (!fwd) {
@@ -459,10 +421,10 @@ __global__ void __launch_bounds__(pass_threads(Sh::EL, sizeof(T))) col_kernel(Ge
         }
       }
     } else {
-      C* tile = fb.take();
+      C* out = fb.take();
       if (fb.active) {
 #pragma unroll
-        for (int m = 0; m < EL; ++m) QG_ST(tile, t + sh.tt() * m, fb.len, st, x[m]);
+        for (int m = 0; m < EL; ++m) QG_ST(out, t + sh.tt() * m, fb.len, st, x[m]);
       }
       __syncthreads();
       const int par = cf.one_buf ? 0 : fb.ph ^ 1;  // parity of the tiles' buffers
@@ -483,12 +445,13 @@ cudaError_t launch_col_shape(const Geom& g, const FftPlan& plan, const Sh& sh, c
                              cudaStream_t st) {
   const ColConfig c = col_config(g, plan, d, W, (int)sizeof(T));
   const auto* twp = reinterpret_cast<const cplx_t<T>*>(tw);
-  const dim3 grid(g.Kcp / W), block(c.threads);
+  const dim3 grid(c.grid), block(c.threads);
+  const ColScalars<T> cs = col_scalars<T>(g, d);
 #define QG_COL_P(P)                                                           \
   case P: {                                                                   \
     const cudaError_t e = raise_smem_limit<col_kernel<T, Sh, P>>(c.smem);     \
     if (e != cudaSuccess) return e;                                           \
-    return launch_pdl(d.pdl != 0, col_kernel<T, Sh, P>, grid, block, c.smem, st, g, sh, c, d, twp); \
+    return launch_pdl(d.pdl != 0, col_kernel<T, Sh, P>, grid, block, c.smem, st, g, sh, c, d, cs, twp); \
   }
   switch (d.op) {
     QG_COL_P(CO_DERIVE)

@@ -8,6 +8,7 @@
 
 #include "fast.cuh"
 #include "qg_kernels.h"
+#include "spectral.cuh"
 #include "tma.cuh"
 
 #ifndef QG_COL_MINB
@@ -31,16 +32,17 @@ namespace fast {
 
 template <int N> struct RowCfg {
   static constexpr int TT = Eng<float, N>::TT;
-  // whole rows, a divisor of N, filling at most QG_ROW_CTA_THREADS threads
-  static constexpr int rows(int r) { return r <= 1 ? 1 : N % r == 0 ? r : rows(r - 1); }
+  // groups of TT threads, each with a row (or two rows that share a transform), filling at most QG_ROW_CTA_THREADS threads
+  static constexpr int rows(int r) { return r <= 1 ? 1 : N % (2 * r) == 0 ? r : rows(r - 1); }
   static constexpr int ROWS = rows(QG_ROW_CTA_THREADS / TT);
   static constexpr int THREADS = TT * ROWS;
 };
 // Resident CTAs per SM requested from the register allocator: 512 threads an SM leave each thread 128 registers, which
-// the row programs and the column ops need (384 with eighteen elements per thread).  Asking for four row CTAs and two
+// the row programs and the column ops need (the rows with twelve or eighteen elements per thread take 168: Smagorinsky
+// rows at 1296^2 38.3 us against 42.6).  Asking for four row CTAs and two
 // column CTAs whatever their size left 64 registers at 4096^2, and a Leith step there took 2.06 ms instead of 1.39.
 template <int N> constexpr int row_occ() {
-  const int target = Eng<float, N>::EL == 18 ? 384 : 512;
+  const int target = Eng<float, N>::EL == 16 || Eng<float, N>::EL == 8 ? 512 : 384;
   return target / RowCfg<N>::THREADS > 0 ? target / RowCfg<N>::THREADS : 1;
 }
 template <int N> constexpr int col_threads();
@@ -115,6 +117,8 @@ struct RowCtx {
   const C* tw;  // per-pass twiddle table
   const Geom* g;
   int bad;
+  int stop;     // the status flag, loaded at the start
+  bool first;   // it has not been looked at yet
 
   // inverse x-transform of the pair a + i b of half-spectrum rows given by f(k, a, b), k <= K
   template <typename F> __device__ __forceinline__ void inv_pair_of(C* x, F f) {
@@ -135,17 +139,28 @@ struct RowCtx {
       }
       x[m] = z;
     }
+    look<true>();
     E::run(x, t, b0, b1, ph, tw, +1);
   }
 
-  __device__ __forceinline__ const C* mixed_row(const void* A) const {
-    return reinterpret_cast<const C*>(A) + (size_t)y * g->IP;
+  // leave if the status flag was set: on small grids after the first inputs' loads are on their way, which hides the
+  // flag's own load; larger ones hide it behind their other CTAs and look at once (LATE: a call with loads under way)
+  static constexpr bool kLate = N < 1024;
+  template <bool LATE> __device__ __forceinline__ void look() {
+    if constexpr (LATE == kLate) {
+      if (first && __syncthreads_or(stop)) leave();
+      first = false;
+    }
   }
 
-  // inverse x-transform of the pair (A + i B) of half-spectrum rows; B may be null
-  __device__ __forceinline__ void inv_pair(C* x, const void* Av, const void* Bv) {
+  __device__ __forceinline__ const C* mixed_row(const void* A, int dy = 0) const {
+    return reinterpret_cast<const C*>(A) + (size_t)(y + dy) * g->IP;
+  }
+
+  // inverse x-transform of the pair (A + i B) of half-spectrum rows; B may be null, or of the next row (dyb = 1)
+  __device__ __forceinline__ void inv_pair(C* x, const void* Av, const void* Bv, int dyb = 0) {
     const C* A = mixed_row(Av);
-    const C* B = Bv ? mixed_row(Bv) : nullptr;
+    const C* B = Bv ? mixed_row(Bv, dyb) : nullptr;
     inv_pair_of(x, [&](int k, C& a, C& b) {
       a = A[k];
       b = B ? B[k] : mk<C>(T(0), T(0));
@@ -153,22 +168,24 @@ struct RowCtx {
   }
 
   // forward x-transform of (re, im) = two real rows, split, optional i k_x, store kept columns
-  __device__ __forceinline__ void fwd_store(C* x, void* Av, void* Bv, bool dxa, bool dxb) {
+  // yb: row of the second output (default: this row)
+  __device__ __forceinline__ void fwd_store(C* x, void* Av, void* Bv, bool dxa, bool dxb, int ya = -1, int yb = -1) {
+    look<true>();
     E::run(x, t, b0, b1, ph, tw, -1);
-    split_store(x, Av, Bv, dxa, dxb);
+    split_store(x, Av, Bv, dxa, dxb, ya < 0 ? y : ya, yb < 0 ? y : yb);
   }
 
   // split the forward transform of two real rows (re, im) into their half spectra, optional i k_x, store the
   // kept columns
-  __device__ __forceinline__ void split_store(C* x, void* Av, void* Bv, bool dxa, bool dxb) {
+  __device__ __forceinline__ void split_store(C* x, void* Av, void* Bv, bool dxa, bool dxb, int ya, int yb) {
     C* ub = ph ? b1 : b0;
     ph ^= 1;
 #pragma unroll
     for (int m = 0; m < E::EL; ++m) ub[E::pad(t + TT * m)] = x[m];
     __syncthreads();
-    C* A = reinterpret_cast<C*>(Av) + (size_t)y * g->IP;
-    C* B = Bv ? reinterpret_cast<C*>(Bv) + (size_t)y * g->IP : nullptr;
-    const T ks = T(g->kscale);
+    C* A = reinterpret_cast<C*>(Av) + (size_t)ya * g->IP;
+    C* B = Bv ? reinterpret_cast<C*>(Bv) + (size_t)yb * g->IP : nullptr;
+    const T ks = g->kscale_f;
 #pragma unroll
     for (int m = 0; m < E::EL; ++m) {
       const int k = t + TT * m;
@@ -216,7 +233,7 @@ __device__ __forceinline__ void level_products(RowCtx<T, N>& cx, cplx_t<T>* x, c
     P[m] = x[m].y;  // v
   }
   if constexpr (SMAG) {
-    const T ks = T(cx.g->kscale);
+    const T ks = cx.g->kscale_f;
     const C *u = cx.mixed_row(in[0]), *v = cx.mixed_row(in[1]), *w = cx.mixed_row(in[2]), *wy = cx.mixed_row(in[3]);
     cx.inv_pair_of(x, [&](int k, C& a, C& b) {  // (w_x, w_y)
       a = cmul_ik(w[k], ks * T(k));
@@ -270,16 +287,19 @@ __global__ void __launch_bounds__(RowCfg<N>::THREADS, row_occ<N>()) row_fast_ker
   const int lr = threadIdx.x / TT;
   RowCtx<T, N> cx;
   cx.t = threadIdx.x % TT;
-  cx.y = blockIdx.x * RowCfg<N>::ROWS + lr;
+  // one field alone to scale or copy: two rows share a transform
+  const bool lone = PROG == RP_SCALE ? d.nin == 1
+                    : PROG == RP_COPY ? d.npair == 0 && (d.in_phys ? !d.phys_in2 : !d.phys_out2) : false;
+  cx.y = (blockIdx.x * RowCfg<N>::ROWS + lr) * (lone ? 2 : 1);
   cx.b0 = sm + (size_t)(2 * lr) * E::BUF;
   cx.b1 = cx.b0 + E::BUF;
   cx.ph = 0;
   cx.tw = tw;
   cx.g = &g;
   cx.bad = 0;
-  if (d.flag) {
-    if (__syncthreads_or(*reinterpret_cast<volatile int*>(d.flag) != 0)) return;
-  }
+  cx.stop = d.flag ? *reinterpret_cast<volatile int*>(d.flag) : 0;
+  cx.first = true;
+  cx.template look<false>();
   const int t = cx.t;
   const size_t yN = (size_t)cx.y * N;
   C x[E::EL];
@@ -288,7 +308,6 @@ __global__ void __launch_bounds__(RowCfg<N>::THREADS, row_occ<N>()) row_fast_ker
     constexpr bool smag = PROG == RP_SMAG || PROG == RP_DSMAG;
     constexpr bool dyn = PROG == RP_DLEITH || PROG == RP_DSMAG;
     constexpr bool none = PROG == RP_NONE;
-    constexpr int per = 4;  // inputs per level
     T J[E::EL], P[E::EL], Q[E::EL];
     level_products<T, N, smag, none>(cx, x, d.in + 0, J, P, Q);
     if constexpr (none) {
@@ -308,7 +327,7 @@ __global__ void __launch_bounds__(RowCfg<N>::THREADS, row_occ<N>()) row_fast_ker
         T Qk[E::EL];
 #pragma unroll
         for (int m = 0; m < E::EL; ++m) Qk[m] = Q[m];
-        level_products<T, N, smag, false>(cx, x, d.in + per, J, P, Q);
+        level_products<T, N, smag, false>(cx, x, d.in + 4, J, P, Q);
 #pragma unroll
         for (int m = 0; m < E::EL; ++m) x[m] = mk<C>(Qk[m], Q[m]);
         cx.fwd_store(x, d.out[2], d.out[5], false, false);
@@ -318,16 +337,16 @@ __global__ void __launch_bounds__(RowCfg<N>::THREADS, row_occ<N>()) row_fast_ker
       }
     }
   } else if constexpr (PROG == RP_SCALE) {
-    // Brinkman (2 fields) or sponge (1 field): multiply by the exact factor field
+    // Brinkman (2 fields) or sponge (1 field, two rows): multiply by the exact factor field
     const T* fac = reinterpret_cast<const T*>(d.factor) + yN;
-    cx.inv_pair(x, d.in[0], d.nin > 1 ? d.in[1] : nullptr);
+    const T* fac2 = lone ? fac + N : fac;
+    cx.inv_pair(x, d.in[0], lone ? d.in[0] : d.in[1], lone);
 #pragma unroll
     for (int m = 0; m < E::EL; ++m) {
-      const T f = fac[t + TT * m];
-      x[m] = mk<C>(x[m].x * f, x[m].y * f);
+      x[m] = mk<C>(x[m].x * fac[t + TT * m], x[m].y * fac2[t + TT * m]);
       cx.bad |= !isfinite(x[m].x) | !isfinite(x[m].y);
     }
-    cx.fwd_store(x, d.out[0], d.nout > 1 ? d.out[1] : nullptr, false, false);
+    cx.fwd_store(x, d.out[0], lone ? d.out[0] : d.out[1], false, false, cx.y, cx.y + lone);
   } else if constexpr (PROG == RP_ADJ_FWD) {
     // one stage of the step recomputed for its adjoint: inverse transforms of (u_total, v), (w_x, w_y)
     // [, (psi_xy, psi_d)], which are kept as physical fields, then J, g w_x, g w_y (Eq. 1, 9, 10, 13) forward
@@ -458,22 +477,21 @@ __global__ void __launch_bounds__(RowCfg<N>::THREADS, row_occ<N>()) row_fast_ker
         }
       }
     }
-  } else {  // RP_COPY: one or two physical rows in or out (two as the real and imaginary parts of one FFT)
+  } else {  // RP_COPY: two physical rows in or out, of two fields or of one (as the real and imaginary parts of one FFT)
     if (d.in_phys) {
       const T* src = reinterpret_cast<const T*>(d.phys_in) + yN;
-      const T* src2 = d.phys_in2 ? reinterpret_cast<const T*>(d.phys_in2) + yN : nullptr;
+      const T* src2 = lone ? src + N : reinterpret_cast<const T*>(d.phys_in2) + yN;
 #pragma unroll
-      for (int m = 0; m < E::EL; ++m) x[m] = mk<C>(src[t + TT * m], src2 ? src2[t + TT * m] : T(0));
-      cx.fwd_store(x, d.out[0], src2 ? d.out[1] : nullptr, false, false);
+      for (int m = 0; m < E::EL; ++m) x[m] = mk<C>(src[t + TT * m], src2[t + TT * m]);
+      cx.fwd_store(x, d.out[0], lone ? d.out[0] : d.out[1], false, false, cx.y, cx.y + lone);
     } else {
-      cx.inv_pair(x, d.in[0], d.phys_out2 ? d.in[1] : nullptr);
+      cx.inv_pair(x, d.in[0], lone ? d.in[0] : d.in[1], lone);
       T* dst = reinterpret_cast<T*>(d.phys_out) + yN;
+      T* dst2 = lone ? dst + N : reinterpret_cast<T*>(d.phys_out2) + yN;
 #pragma unroll
-      for (int m = 0; m < E::EL; ++m) dst[t + TT * m] = x[m].x;
-      if (d.phys_out2) {
-        T* dst2 = reinterpret_cast<T*>(d.phys_out2) + yN;
-#pragma unroll
-        for (int m = 0; m < E::EL; ++m) dst2[t + TT * m] = x[m].y;
+      for (int m = 0; m < E::EL; ++m) {
+        dst[t + TT * m] = x[m].x;
+        dst2[t + TT * m] = x[m].y;
       }
     }
   }
@@ -485,18 +503,6 @@ __global__ void __launch_bounds__(RowCfg<N>::THREADS, row_occ<N>()) row_fast_ker
 // ---------------------------------------------------------------------------
 // Column pass
 // ---------------------------------------------------------------------------
-template <typename T> struct FInvK2;
-template <> struct FInvK2<double> {
-  __device__ static double get(double ks2, int m2) { return m2 == 0 ? 0.0 : 1.0 / (ks2 * double(m2)); }
-};
-template <> struct FInvK2<float> {
-  __device__ static float get(double ks2, int m2) {
-    if (m2 == 0) return 0.f;
-    if (m2 <= 16) return float(1.0 / (ks2 * double(m2)));
-    return 1.f / (float(ks2) * float(m2));
-  }
-};
-
 // modes per batch in the column pass's state update (loads of a batch precede its stores)
 #ifndef QG_STATE_BATCH
 #define QG_STATE_BATCH 8
@@ -508,7 +514,8 @@ constexpr int kStateBatch = QG_STATE_BATCH;
 // a partial second wave of column CTAs into one wave.
 template <typename T, int N, int OP, bool LEAN = false>
 __global__ void __launch_bounds__(ColCfg<N>::THREADS, LEAN ? 3 : Occ<OP, N>::col) col_fast_kernel(
-    Geom g, ColDesc d, const cplx_t<T>* __restrict__ tw, const __grid_constant__ TmaSet tm) {
+    Geom g, ColDesc d, const __grid_constant__ ColScalars<T> cs, const cplx_t<T>* __restrict__ tw,
+    const __grid_constant__ TmaSet tm) {
   pdl_enter();
   using E = Eng<T, N>;
   using C = cplx_t<T>;
@@ -542,9 +549,7 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, LEAN ? 3 : Occ<OP, N>::col
   const bool lead = threadIdx.x == 0;
   int ph = 0;
   const C* twb = tw;
-  if (d.flag) {
-    if (__syncthreads_or(*reinterpret_cast<volatile int*>(d.flag) != 0)) return;
-  }
+  const int stop = d.flag ? *reinterpret_cast<volatile int*>(d.flag) : 0;
   // thread 0 starts the first NSTG forward fields' tiles
   if (lead) {
     tma::mbar_init(&mbar[0], 1);
@@ -564,10 +569,19 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, LEAN ? 3 : Occ<OP, N>::col
       }
     }
   }
-  __syncthreads();
-  const double ks2 = g.kscale * g.kscale;
-  const double n2 = double(N) * double(N);
-  const T kxv = T(g.kscale) * T(mx);
+  // the status flag's load has overlapped the tiles' requests
+  if constexpr (OP != CO_DYN_COMBINE && OP != CO_AB2CN_COMBINE) {
+    if (__syncthreads_or(stop)) {
+      if constexpr (OP != CO_DERIVE) {
+        // leave once no tile is in flight
+        if (lead && (int)blockIdx.x + 1 != d.stall_cta1)
+          for (int f = 0; f < d.nfwd && f < NSTG; ++f) tma::mbar_wait(&mbar[f], 0, kWaitCycles);
+        __syncthreads();
+      }
+      return;
+    }
+  }
+  const T kxv = cs.ks * T(mx);
   C* w0 = reinterpret_cast<C*>(d.w0);
   C* ws = reinterpret_cast<C*>(d.ws);
   C* jh = reinterpret_cast<C*>(d.jh);
@@ -639,7 +653,7 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, LEAN ? 3 : Occ<OP, N>::col
             const int k = t + TT * m;
             if (!(k <= K || k >= N - K) || !act) continue;
             const int my = k <= K ? k : k - N;
-            const T ky = T(g.kscale) * T(my);
+            const T ky = cs.ks * T(my);
             const size_t gi = colbase + (k <= K ? k : k - N + Ny);
             const bool in_test = mx * mx + my * my <= d.test_m2max;
             const C X = col_ok ? x[m] : mk<C>(T(0), T(0));
@@ -654,13 +668,13 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, LEAN ? 3 : Occ<OP, N>::col
             } else if (f == 3) {
               s2[gi] = in_test ? csub(X, la[q]) : X;
             } else if (f == 4) {
-              s1[gi] = cadd(la[q], cscale(X, T(d.rpow)));
+              s1[gi] = cadd(la[q], cscale(X, cs.rpow));
             } else if (f == 6) {
-              s0[gi] = cscale(cmul_ik(X, ky), T(d.inv_eta));
+              s0[gi] = cscale(cmul_ik(X, ky), cs.inv_eta);
             } else if (f == 7) {
-              reinterpret_cast<C*>(d.bh)[gi] = csub(la[q], cscale(cmul_ik(X, kxv), T(d.inv_eta)));
+              reinterpret_cast<C*>(d.bh)[gi] = csub(la[q], cscale(cmul_ik(X, kxv), cs.inv_eta));
             } else if (col_ok) {
-              const C M = cadd(la[q], cscale(cmul_ik(X, ky), T(d.rpow)));
+              const C M = cadd(la[q], cscale(cmul_ik(X, ky), cs.rpow));
               const C H = lb[q];
               const T wgt = mx == 0 ? T(1) : T(2);
               acc_hm.add_prod(wgt * H.x, M.x);
@@ -675,7 +689,7 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, LEAN ? 3 : Occ<OP, N>::col
       for (int m = 0; m < E::EL && !LEAN; ++m) {
         const int k = t + TT * m;
         const int my = k <= K ? k : k - N;
-        const T ky = T(g.kscale) * T(my);
+        const T ky = cs.ks * T(my);
         C X = col_ok ? x[m] : mk<C>(T(0), T(0));
         if constexpr (OP == CO_STAGE_STATIC) {
           if (f == 0) A[m] = mk<C>(-X.x, -X.y);
@@ -697,14 +711,14 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, LEAN ? 3 : Occ<OP, N>::col
           } else if (f == 3) {
             A[m] = in_test ? csub(X, A[m]) : X;
           } else if (f == 4) {
-            B[m] = cadd(B[m], cscale(X, T(d.rpow)));
+            B[m] = cadd(B[m], cscale(X, cs.rpow));
           } else if (f == 6) {  // Brinkman pair (paper's scheme): F_obs = (i ky F[chi u] - i kx F[chi v]) / eta
-            A[m] = cscale(cmul_ik(X, ky), T(d.inv_eta));
+            A[m] = cscale(cmul_ik(X, ky), cs.inv_eta);
           } else if (f == 7) {
-            A[m] = csub(A[m], cscale(cmul_ik(X, kxv), T(d.inv_eta)));
+            A[m] = csub(A[m], cscale(cmul_ik(X, kxv), cs.inv_eta));
             if (kept) reinterpret_cast<C*>(d.bh)[colbase + r] = A[m];
           } else {
-            const C M = cadd(B[m], cscale(cmul_ik(X, ky), T(d.rpow)));
+            const C M = cadd(B[m], cscale(cmul_ik(X, ky), cs.rpow));
             const C H = A[m];
             if (kept && col_ok) {
               // weight 2 for k_x > 0 (the conjugate half), applied exactly
@@ -722,8 +736,8 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, LEAN ? 3 : Occ<OP, N>::col
           // E = -J + C D + F_obs: A collects -J + F_obs, B collects D
           if (f == 0) A[m] = mk<C>(-X.x, -X.y);
           else if (f < d.nst) B[m] = (f == 1) ? X : cadd(B[m], cmul_ik(X, ky));
-          else if (f == d.nst) A[m] = cadd(A[m], cscale(cmul_ik(X, ky), T(d.inv_eta)));
-          else A[m] = csub(A[m], cscale(cmul_ik(X, kxv), T(d.inv_eta)));
+          else if (f == d.nst) A[m] = cadd(A[m], cscale(cmul_ik(X, ky), cs.inv_eta));
+          else A[m] = csub(A[m], cscale(cmul_ik(X, kxv), cs.inv_eta));
         } else if constexpr (OP == CO_FORWARD2) {
           if (f == 0) A[m] = X;
           else B[m] = X;
@@ -743,6 +757,7 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, LEAN ? 3 : Occ<OP, N>::col
   if constexpr (OP == CO_FORWARD_N) {
     return;  // every field's band is stored; no state update, no derived fields, no bulk stores in flight
   } else if constexpr (OP == CO_DYN_REDUCE) {
+    // (pair_sum's form of this costs registers throughout the loop above: 62.6 against 53.3 us at 2048^2)
     double hm = acc_hm.value(), mm = acc_mm.value();
     for (int o = 16; o > 0; o >>= 1) {
       hm += __shfl_down_sync(0xffffffffu, hm, o);
@@ -769,25 +784,9 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, LEAN ? 3 : Occ<OP, N>::col
     }
     return;
   } else {
-    T coeff = T(d.coeff);
+    T coeff = cs.coeff;
     if constexpr (OP == CO_DYN_COMBINE || OP == CO_AB2CN_COMBINE) {
-      if (threadIdx.x < 32) {
-        double a = 0.0, b = 0.0;
-        for (int i = threadIdx.x; i < d.npartials; i += 32) {
-          a += d.partials[2 * i];
-          b += d.partials[2 * i + 1];
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-          a += __shfl_down_sync(0xffffffffu, a, o);
-          b += __shfl_down_sync(0xffffffffu, b, o);
-        }
-        if (threadIdx.x == 0) {
-          const double Cc = b > 0.0 ? fmax(0.0, a / b) : 0.0;
-          red[0][0] = Cc;
-          if (blockIdx.x == 0 && d.coeff_out) *d.coeff_out = Cc;
-        }
-      }
-      __syncthreads();
+      if (!germano_coefficient(d.partials, d.npartials, red, ColCfg<N>::THREADS, stop, d.coeff_out, nullptr)) return;
       coeff = T(red[0][0]);
     }
 
@@ -795,10 +794,10 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, LEAN ? 3 : Occ<OP, N>::col
     // of GB whose global loads are all issued before any of the batch's
     // stores: the state arrays may alias as far as the compiler can tell, so
     // a load placed after a store would wait for that store's round trip.
-    const T dt = T(d.dt), a_rk = T(d.a), b_rk = T(d.b), beta = T(d.beta);
+    const T dt = cs.dt, a_rk = cs.a, b_rk = cs.b, beta = cs.beta;
     const T* vx = reinterpret_cast<const T*>(d.visc_x);
     const T* vy = reinterpret_cast<const T*>(d.visc_y);
-    const T vmu = T(d.visc_mu);
+    const T vmu = cs.visc_mu;
     const C* bhp = reinterpret_cast<const C*>(d.bh);
     C* ep = reinterpret_cast<C*>(d.eprev);
     C* wsp = reinterpret_cast<C*>(d.wss);
@@ -861,7 +860,7 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, LEAN ? 3 : Occ<OP, N>::col
           } else if constexpr (OP == CO_STAGE_STATIC || OP == CO_DYN_COMBINE) {
             const C wz = u0[q];
             const C wst = u1[q];
-            const T ik2 = FInvK2<T>::get(ks2, mx * mx + my * my);
+            const T ik2 = inv_k2<T>(cs, mx * mx + my * my);
             const C psi = mk<C>(-wst.x * ik2, -wst.y * ik2);
             const C bv = cscale(cmul_ik(psi, kxv), beta);
             C L;
@@ -886,10 +885,10 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, LEAN ? 3 : Occ<OP, N>::col
             const C Ep = d.ab2_first ? E : u1[q];
             ep[gi] = E;
             const int m2 = mx * mx + my * my;
-            const T k2 = T(ks2) * T(m2);
-            const T ik2 = FInvK2<T>::get(ks2, m2);
+            const T k2 = cs.ks2 * T(m2);
+            const T ik2 = inv_k2<T>(cs, m2);
             const T hdt = T(0.5) * dt;
-            const T lre = -(T(d.nu) * k2 + T(d.mu));
+            const T lre = -(cs.nu * k2 + cs.mu);
             const T lim = beta * kxv * ik2;
             const C wz = u0[q];
             const C ab = mk<C>(T(1.5) * E.x - T(0.5) * Ep.x, T(1.5) * E.y - T(0.5) * Ep.y);
@@ -928,7 +927,7 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, LEAN ? 3 : Occ<OP, N>::col
     // Per owned mode: the state scaled by 1/N^2 (so the two inverse passes
     // return physical values), 1/|k|^2, and masks of the kept 2/3 band and of
     // the test filter; each derived field then costs a few operations per mode.
-    const T scale = T(1.0 / n2);
+    const T scale = cs.scale;
     T ik2[E::EL];
     unsigned keep = 0u, intest = 0u;
 #pragma unroll
@@ -938,10 +937,10 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, LEAN ? 3 : Occ<OP, N>::col
       const int m2 = mx * mx + my * my;
       if ((k <= K || k >= N - K) && col_ok) keep |= 1u << m;
       if (m2 <= d.test_m2max) intest |= 1u << m;
-      ik2[m] = FInvK2<T>::get(ks2, m2);
+      ik2[m] = inv_k2<T>(cs, m2);
       A[m] = cscale(A[m], scale);
     }
-    const T ksc = T(g.kscale);
+    const T ksc = cs.ks;
     // Three shared buffers rotate between the transform's two exchange buffers and the output tile of the TMA
     // store: the tile goes to the exchange buffer the transform's last exchange did not use (so no barrier is
     // needed before it is written), and the next field avoids the buffer whose store may still be reading.
@@ -964,7 +963,7 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, LEAN ? 3 : Occ<OP, N>::col
         case D_U:  // -i ky psi, psi = -w / |k|^2
 #pragma unroll
           for (int m = 0; m < E::EL; ++m) x[m] = cmul_ik(cscale(w[m], ik2[m]), QG_KY(m));
-          if (mx == 0 && t == 0) x[0] = mk<C>(T(d.U), T(0));
+          if (mx == 0 && t == 0) x[0] = mk<C>(cs.U, T(0));
           break;
         case D_V:  // i kx psi
 #pragma unroll
@@ -1035,13 +1034,15 @@ cudaError_t launch_row_fast(const Geom& g, const RowDesc& d, const void* tw, cud
   using Cfg = fast::RowCfg<N>;
   const size_t smem = (size_t)2 * Cfg::ROWS * E::BUF * sizeof(cplx_t<T>);
   const auto* twp = reinterpret_cast<const cplx_t<T>*>(tw);
-  const int grid = N / Cfg::ROWS;
+  const bool lone = d.prog == RP_SCALE ? d.nin == 1
+                    : d.prog == RP_COPY ? d.npair == 0 && (d.in_phys ? !d.phys_in2 : !d.phys_out2) : false;
   cudaError_t e = cudaSuccess;
 #define QG_ROW_CASE(P)                                                                                   \
   case P: {                                                                                              \
     auto k = fast::row_fast_kernel<T, N, P>;                                                            \
     e = raise_smem_limit<fast::row_fast_kernel<T, N, P>>(smem);                                          \
     if (e != cudaSuccess) return e;                                                                      \
+    const int grid = N / Cfg::ROWS / (lone ? 2 : 1);                                                         \
     e = launch_pdl(d.pdl != 0, k, dim3(grid), dim3(Cfg::THREADS), smem, st, g, d, twp);                \
     if (e != cudaSuccess) return e;                                                                      \
     break;                                                                                               \
@@ -1066,12 +1067,13 @@ cudaError_t launch_row_fast(const Geom& g, const RowDesc& d, const void* tw, cud
 template <typename T, int N, int P, bool LEAN>
 cudaError_t launch_col_one(const Geom& g, const ColDesc& d, const cplx_t<T>* twp, const TmaSet& tm, int grid,
                            cudaStream_t st) {
+  const ColScalars<T> cs = col_scalars<T>(g, d);
   using Cfg = fast::ColCfg<N>;
   auto k = fast::col_fast_kernel<T, N, P, LEAN>;
   const size_t smem = (size_t)(LEAN ? 2 : 3) * fast::col_stage_bytes<T, N>() + 1024;
   const cudaError_t e = raise_smem_limit<fast::col_fast_kernel<T, N, P, LEAN>>(smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(d.pdl != 0, k, dim3(grid), dim3(Cfg::THREADS), smem, st, g, d, twp, tm);
+  return launch_pdl(d.pdl != 0, k, dim3(grid), dim3(Cfg::THREADS), smem, st, g, d, cs, twp, tm);
 }
 
 // SMs of the current device, queried once per device (concurrent first calls store the same value)

@@ -375,16 +375,21 @@ template <typename C> __device__ __forceinline__ void bfly(C& a, C& b, C w) {
 // Butterfly of radix R with its twiddles w[(r - 1) ns] (kernel exp(s 2 pi i / N): conjugated for s > 0).  FP64 radices
 // 2 and 4 fuse the twiddles into the butterflies (w v1 + w^3 v3 = w (v1 + w^2 v3)): six FMA-pipe operations per
 // two-point butterfly against eight, and two twiddle loads for radix 4 against three.
-template <typename C, int R, bool PK>
-__device__ __forceinline__ void twiddled(C* v, const C* __restrict__ w, int ns, int s) {
+// GL: the table lies in global memory (else in shared memory or anywhere).
+template <bool GL, typename C> __device__ __forceinline__ C tw_load(const C* w) {
+  if constexpr (GL) return __ldg(w);
+  else return *w;
+}
+template <typename C, int R, bool PK, bool GL>
+__device__ __forceinline__ void twiddled(C* v, const C* w, int ns, int s) {
   using T = decltype(C::x);
   if constexpr (sizeof(T) == 8 && (R == 2 || R == 4)) {
-    C w1 = __ldg(w);
+    C w1 = tw_load<GL>(w);
     if (s > 0) w1.y = -w1.y;
     if constexpr (R == 2) {
       bfly(v[0], v[1], w1);
     } else {
-      C w2 = __ldg(w + ns);
+      C w2 = tw_load<GL>(w + ns);
       if (s > 0) w2.y = -w2.y;
       bfly(v[0], v[2], w2);
       bfly(v[1], v[3], w2);
@@ -397,12 +402,22 @@ __device__ __forceinline__ void twiddled(C* v, const C* __restrict__ w, int ns, 
   } else {
 #pragma unroll
     for (int r = 1; r < R; ++r) {
-      C wr = __ldg(w + (r - 1) * ns);
+      C wr = tw_load<GL>(w + (r - 1) * ns);
       if (s > 0) wr.y = -wr.y;
       v[r] = cmul(v[r], wr);
     }
     dftR<C, R, PK>(v, s);
   }
+}
+
+// The twiddle table of a small plan moves to shared memory at the start of a pass: read from L2 by every pass of
+// every transform it would be most of a short transform's latency.  Larger tables stay in global memory (L1).
+constexpr int kTwShared = 512;  // entries
+__host__ __device__ constexpr bool tw_shared(int table) { return table <= kTwShared; }
+template <typename C> __device__ __forceinline__ const C* tw_stage(const C* tw, int table, C* sm) {
+  if (!tw_shared(table)) return tw;
+  for (int i = threadIdx.x; i < table; i += blockDim.x) sm[i] = __ldg(tw + i);
+  return sm;  // complete at the next CTA barrier
 }
 
 // The run-time transform: EL elements per thread, the plan in a kernel parameter.
@@ -412,10 +427,11 @@ template <int EL_> struct RtShape {
   __device__ __forceinline__ int n() const { return p.n; }
   __device__ __forceinline__ int tt() const { return p.tt; }
   __device__ __forceinline__ int buf() const { return p.buf; }
+  __device__ __forceinline__ int table() const { return p.table; }
   __device__ __forceinline__ int band(const Geom& g) const { return g.K; }
 
   template <int R, typename C>
-  __device__ __forceinline__ void pass(C* x, int t, const FftPass& ps, bool last, C* buf, const C* __restrict__ tw,
+  __device__ __forceinline__ void pass(C* x, int t, const FftPass& ps, bool last, C* buf, const C* tw,
                                        const FftBufs<C>& fb) const {
     constexpr int NB = EL / R;
 #pragma unroll
@@ -428,7 +444,7 @@ template <int EL_> struct RtShape {
       if (ps.ns > 1) {
         q = __umulhi((unsigned)j, ps.inv);
         k = j - q * ps.ns;
-        twiddled<C, R, true>(v, tw + ps.off + k, ps.ns, -1);
+        twiddled<C, R, true, false>(v, tw + ps.off + k, ps.ns, -1);
       } else {
         dftR<C, R, true>(v, -1);
       }
@@ -445,7 +461,7 @@ template <int EL_> struct RtShape {
 
   // forward transform, natural ownership in and out
   template <typename C>
-  __device__ __forceinline__ void run(C* x, int t, FftBufs<C>& fb, const C* __restrict__ tw) const {
+  __device__ __forceinline__ void run(C* x, int t, FftBufs<C>& fb, const C* tw) const {
 #pragma unroll 1
     for (int i = 0; i < p.npass; ++i) {
       const FftPass ps = p.pass[i];
@@ -475,8 +491,8 @@ template <int EL_> struct RtShape {
 
 // Pass I of the compile-time transform of length N: x in natural ownership on entry; a non-last pass writes its
 // outputs to buf (when active), the last one leaves them in x.
-template <typename C, int N, int EL, int I, bool PK>
-__device__ __forceinline__ void st_pass(C* x, int t, C* buf, const C* __restrict__ tw, int s, bool active) {
+template <typename C, int N, int EL, int I, bool PK, bool GL>
+__device__ __forceinline__ void st_pass(C* x, int t, C* buf, const C* tw, int s, bool active) {
   constexpr Radices P = fft_radices(N, EL);
   constexpr int R = P.radix[I], NS = P.ns[I], NB = EL / R, TT = N / EL;
 #pragma unroll
@@ -486,7 +502,7 @@ __device__ __forceinline__ void st_pass(C* x, int t, C* buf, const C* __restrict
     C v[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) v[r] = x[b + NB * r];
-    if constexpr (NS > 1) twiddled<C, R, PK>(v, tw + P.off[I] + k, NS, s);
+    if constexpr (NS > 1) twiddled<C, R, PK, GL>(v, tw + P.off[I] + k, NS, s);
     else dftR<C, R, PK>(v, s);
     if constexpr (I == P.np - 1) {
 #pragma unroll
@@ -505,15 +521,16 @@ template <int N_, int EL_> struct StShape {
   __device__ __forceinline__ constexpr int n() const { return N_; }
   __device__ __forceinline__ constexpr int tt() const { return N_ / EL_; }
   __device__ __forceinline__ constexpr int buf() const { return N_ + N_ / 16 + 1; }
+  __device__ __forceinline__ constexpr int table() const { return fft_radices(N_, EL_).table; }
   __device__ __forceinline__ constexpr int band(const Geom&) const { return (N_ - 1) / 3; }
 
   template <int I, typename C>
-  __device__ __forceinline__ void from(C* x, int t, FftBufs<C>& fb, const C* __restrict__ tw) const {
+  __device__ __forceinline__ void from(C* x, int t, FftBufs<C>& fb, const C* tw) const {
     constexpr int np = fft_radices(N_, EL_).np;
     if constexpr (I < np) {
       constexpr bool last = I == np - 1;
       C* buf = last ? nullptr : fb.take();
-      st_pass<C, N_, EL_, I, true>(x, t, buf, tw, -1, fb.active);
+      st_pass<C, N_, EL_, I, true, false>(x, t, buf, tw, -1, fb.active);
       if constexpr (!last) {
         fb.sync();
 #pragma unroll
@@ -523,7 +540,7 @@ template <int N_, int EL_> struct StShape {
     }
   }
   template <typename C>
-  __device__ __forceinline__ void run(C* x, int t, FftBufs<C>& fb, const C* __restrict__ tw) const {
+  __device__ __forceinline__ void run(C* x, int t, FftBufs<C>& fb, const C* tw) const {
     from<0>(x, t, fb, tw);
   }
 };

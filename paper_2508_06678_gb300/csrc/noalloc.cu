@@ -97,6 +97,7 @@ int run_stats(const void* omega, int n, double L, cudaStream_t st, double* stats
   g.Ny = 2 * g.K + 1;
   g.SP = (g.Ny + 3) / 4 * 4;
   g.kscale = 2.0 * M_PI / L;
+  g.kscale_f = (float)g.kscale;
   const FftPlan plan = fft_plan(n, rt_elems(n, sizeof(T)));
   const int W = col_width(plan, sizeof(T));
   g.Kcp = (g.Kc + W - 1) / W * W;

@@ -18,7 +18,10 @@ FftPlan fft_plan(int n, int el) {
 }
 
 // dynamic shared memory a CTA can have: 227 KB less the passes' static part (under 768 bytes)
+constexpr int kSms = 152;  // of a GB300
 constexpr size_t kSmemCap = 227 * 1024 - 768;
+
+static size_t tw_bytes(const FftPlan& p, int esz) { return tw_shared(p.table) ? (size_t)p.table * 2 * esz : 0; }
 
 RowConfig row_config(const FftPlan& p, const RowDesc& d, int esz) {
   RowConfig c{};
@@ -28,7 +31,7 @@ RowConfig row_config(const FftPlan& p, const RowDesc& d, int esz) {
   c.nslot = direct ? 0 : (nin > nout ? nin : nout);
   auto tasks = [](int rows, int nf) { return rows * (nf / 2) + (nf & 1 ? (rows + 1) / 2 : 0); };
   auto bytes = [&](int rows, int groups, int nbuf) {
-    return (size_t)groups * nbuf * p.buf * 2 * esz + (size_t)rows * c.nslot * p.n * esz;
+    return (tw_bytes(p, esz) + (size_t)groups * nbuf * p.buf * 2 * esz) + (size_t)rows * c.nslot * p.n * esz;
   };
   const bool odd = (nin & 1) || (nout & 1);
   c.rows = odd && (direct || (p.n >= 256 && bytes(2, 1, 2) <= kSmemCap / 2)) ? 2 : 1;
@@ -46,6 +49,11 @@ RowConfig row_config(const FftPlan& p, const RowDesc& d, int esz) {
   if (c.rows == 2 && bytes(2, groups, 1) > kSmemCap) c.rows = 1;
   c.smem = bytes(c.rows, groups, c.one_buf ? 1 : 2);
   c.threads = (groups * p.tt + 31) / 32 * 32;
+  // FP64 is bound by its operations, so the last, partial round of row pairs goes out as single rows where that
+  // leaves no SM with two of them (1024^2: 3 pairs and a row per SM against 4 pairs)
+  const int pairs = p.n / c.rows, rest = pairs % kSms;
+  c.full = pairs;
+  if (esz == 8 && c.rows == 2 && !direct && pairs > kSms && rest > 0 && 2 * rest <= kSms) c.full = pairs - rest;
   c.warp = p.tt <= 32 && 32 % p.tt == 0;
   return c;
 }
@@ -61,7 +69,7 @@ ColConfig col_config(const Geom& g, const FftPlan& p, const ColDesc& d, int W, i
   c.pitch = (p.buf + 15) / 16 * 16 + (W > 1 ? (esz == 4 ? 16 : 8) / W : 0);
   const int most = d.nfwd > d.nder ? d.nfwd : d.nder;
   auto bytes = [&](int f, int nbuf) {
-    return ((size_t)f * W * nbuf * c.pitch + 2 * (size_t)W * g.Ny) * 2 * esz;
+    return tw_bytes(p, esz) + ((size_t)f * W * nbuf * c.pitch + 2 * (size_t)W * g.Ny) * 2 * esz;
   };
   const int target = esz == 4 ? 256 : 192;
   int f = target / (p.tt * W);
@@ -74,6 +82,25 @@ ColConfig col_config(const Geom& g, const FftPlan& p, const ColDesc& d, int W, i
   c.one_buf = bytes(f, 2) > kSmemCap;
   c.smem = bytes(f, c.one_buf ? 1 : 2);
   c.threads = (f * W * p.tt + 31) / 32 * 32;
+  // FP64: the columns beyond a whole number of rounds over the SMs share out their outgoing fields, one CTA per SM,
+  // at the price of transforming the incoming ones in each (1024^2: 342 columns, 38 of them in four parts; with the
+  // single rows of row_config 1508 -> 1374 us per step).  Not with less than a round: 128^2, 43 columns in three
+  // parts each, 140 us against 136.  Not where an op reads what it writes: a column's parts run at the same time.
+  const int tiles = g.Kcp / W, rest = tiles % kSms;
+  bool reads_own = d.op == CO_AB2CN || d.op == CO_AB2CN_COMBINE ||
+                   ((d.op == CO_STAGE_STATIC || d.op == CO_DYN_COMBINE) && d.store_w0);
+  for (int i = 0; i < d.nfwd; ++i)
+    for (int q = 0; q < d.nder; ++q) reads_own = reads_own || d.fin[i] == d.dout[q];
+  c.full = tiles;
+  c.split = 1;
+  if (esz == 8 && !reads_own && d.nder > 1 && rest > 0 && tiles > kSms) {
+    const int s = kSms / rest < d.nder ? kSms / rest : d.nder;
+    if (s > 1) {
+      c.split = s;
+      c.full = tiles - rest;
+    }
+  }
+  c.grid = c.full + (tiles - c.full) * c.split;
   c.warp = p.tt * W <= 32 && 32 % (p.tt * W) == 0;
   return c;
 }

@@ -161,6 +161,8 @@ struct qg_handle {
   void* ptw = nullptr;  // per-pass twiddle table of the handle's FFT engine
   void* visc_x = nullptr;
   void* visc_y = nullptr;
+  void* ik2 = nullptr;      // FP64: 1 / |k|^2 per stored mode
+  void* adj_ik2 = nullptr;  // the same for an FP32 handle's adjoint, which combines spectra in FP64
   void* phys = nullptr;
   double visc_mu = 1.0;
   double* partials = nullptr;  // Germano partial sums (2 per column block)
@@ -174,6 +176,7 @@ struct qg_handle {
   // launch forms of the step chosen by an ensemble's tuner: programmatic dependent launch, the FP32 Germano
   // reduction's lean form (ColDesc::lean); both leave the arithmetic unchanged
   int step_pdl = 0;
+  int adj_pdl = 1;  // the adjoint's passes launch programmatically
   int lean_reduce = 0;
   cudaEvent_t flag_event = nullptr;
   bool flag_pending = false;
@@ -272,6 +275,25 @@ int upload_real(qg_handle* h, void* dst, const std::vector<double>& v) {
   return QG_OK;
 }
 
+int upload_f64(qg_handle* h, void* dst, const std::vector<double>& v) {
+  CK(cudaMemcpyAsync(dst, v.data(), v.size() * 8, cudaMemcpyHostToDevice, h->stream), "upload");
+  CK(cudaStreamSynchronize(h->stream), "upload sync");
+  return QG_OK;
+}
+
+// 1 / |k|^2 of every stored mode (0 for the mean mode and the padding), FP64
+int upload_ik2(qg_handle* h, void** out) {
+  const Geom& g = h->g;
+  std::vector<double> ik((size_t)g.Kcp * g.SP, 0.0);
+  for (int c = 0; c < g.Kc; ++c)
+    for (int r = 0; r < g.Ny; ++r) {
+      const int my = my_of_r(g, r), m2 = c * c + my * my;
+      if (m2) ik[(size_t)c * g.SP + r] = 1.0 / (g.kscale * g.kscale * double(m2));
+    }
+  const int rc = dalloc(h, out, ik.size() * 8);
+  return rc ? rc : upload_f64(h, *out, ik);
+}
+
 cudaEvent_t take_event(qg_handle* h) {
   if (!h->pool.empty()) {
     cudaEvent_t e = h->pool.back();
@@ -350,7 +372,7 @@ cudaError_t col_dispatch(qg_handle* h, const ColDesc& d) {
 int run_row(qg_handle* h, RowDesc& d, int cls, bool use_flag = true) {
   d.flag = use_flag ? h->flag : nullptr;
   d.err = h->flag;
-  if (h->step_pdl) d.pdl = 1;
+  d.pdl = (d.pdl && h->adj_pdl) || h->step_pdl;
   Bracket br(h, cls);
   const cudaError_t e = row_dispatch(h, d);
   br.done();
@@ -361,7 +383,7 @@ int run_row(qg_handle* h, RowDesc& d, int cls, bool use_flag = true) {
 int run_col(qg_handle* h, ColDesc& d, int cls, bool use_flag = true) {
   d.flag = use_flag ? h->flag : nullptr;
   d.err = h->flag;
-  if (h->step_pdl) d.pdl = 1;
+  d.pdl = (d.pdl && h->adj_pdl) || h->step_pdl;
   d.lean = h->lean_reduce;
   Bracket br(h, cls);
   const cudaError_t e = col_dispatch(h, d);
@@ -393,6 +415,7 @@ ColDesc col_base(qg_handle* h) {
   d.visc_x = h->visc_x;
   d.visc_y = h->visc_y;
   d.visc_mu = h->visc_mu;
+  d.ik2 = h->ik2;
   d.eprev = h->eprev;
   d.wss = h->wss;
   d.bh = h->bh;
@@ -688,6 +711,7 @@ int adj_alloc(qg_handle* h) {
   for (auto& p : M) if (!rc) rc = dalloc(h, &p, mixed_bytes);
   void* dots = nullptr;
   // partials | dot results (kAdjScalars) | per-stage scalars (4 x 3) | second partials | counter (zeroed here)
+  if (!rc && h->fp32 && !h->adj_ik2) rc = upload_ik2(h, &h->adj_ik2);
   if (!rc) rc = dalloc(h, &dots, sizeof(double) * (2 * kAdjDotBlocks + kAdjScalars + 12 + 1));
   if (!rc && h->fast) {
     const int BR = fast_box_rows(h->g.n);
@@ -856,9 +880,20 @@ int adj_to_phys(qg_handle* h, const void* S, std::initializer_list<int> codes, s
   return rc;
 }
 
+AdjCombine adj_combine_base(const qg_handle* h) {
+  AdjCombine a{};
+  a.ik2 = static_cast<const double*>(h->fp32 ? h->adj_ik2 : h->ik2);
+  if (!h->fp32) {
+    a.visc_x = static_cast<const double*>(h->visc_x);
+    a.visc_y = static_cast<const double*>(h->visc_y);
+    a.visc_mu = h->visc_mu;
+  }
+  return a;
+}
+
 int adj_combine(qg_handle* h, void* out, bool accumulate, bool zero_mean,
                 std::initializer_list<AdjTerm> terms) {
-  AdjCombine a{};
+  AdjCombine a = adj_combine_base(h);
   a.out = out;
   a.accumulate = accumulate;
   a.zero_mean = zero_mean;
@@ -1162,7 +1197,7 @@ int adj_reverse_germano(qg_handle* h, int kind, void* Slam_out, int s) {
     if (rc) return rc;
     const int f = pass == 0 ? AM_TESTF : 0;
     const double sj = pass == 0 ? 1.0 : -1.0, sd = pass == 0 ? rp : -1.0;
-    AdjCombine a{};
+    AdjCombine a = adj_combine_base(h);
     a.out = Slam_out;
     a.accumulate = 1;
     a.test_m2max = h->test_m2max;
@@ -1240,7 +1275,7 @@ int adj_reverse_stage(qg_handle* h, int kind, bool dyn, double C, const void* Sl
   else if (!rc)
     rc = adj_to_spec_many(h, {P[9], P[10], P[11], P[12]}, {S[8], S[9], S[10], S[11]});
   if (rc) return rc;
-  AdjCombine a{};
+  AdjCombine a = adj_combine_base(h);
   a.out = Slam_out;
   a.nu = h->par.nu;
   a.mu = h->par.mu;
@@ -1778,6 +1813,7 @@ int qg_create(const qg_grid* grid, double beta, double U, const double* mask, co
   g.Ny = 2 * g.K + 1;
   g.SP = (g.Ny + 3) / 4 * 4;
   g.kscale = 2.0 * M_PI / grid->L;
+  g.kscale_f = (float)g.kscale;
 
   int dev = 0, smem_optin = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -1827,6 +1863,12 @@ int qg_create(const qg_grid* grid, double beta, double U, const double* mask, co
     const bool generic = getenv("QG_FORCE_GENERIC") != nullptr;
     h->fast = h->fp32 && !generic && fast_grid(n);
     h->wide = h->fp32 && !generic && wide_grid(n);
+    // Programmatic launches hide the start of a step's passes behind the pass before where a pass is a few
+    // microseconds and leaves SMs free; elsewhere the waiting CTAs take room from the running ones.  Measured, us per
+    // step without / with: FP32 64^2 64 / 56, 192^2 102 / 95, 256^2 89 / 84, 324^2 110 / 106, 384^2 83 / 84, 512^2 120 /
+    // 126, 2048^2 681 / 732; FP64 128^2 143 / 136, 256^2 223 / 262.
+    h->step_pdl = n <= (h->fp32 ? 324 : 162) ? 1 : 0;
+    h->adj_pdl = h->fp32 || h->step_pdl;  // FP64 256^2 adjoint step 1.55 ms without, 1.85 with; FP32 0.354 and 0.331
     h->plan = fft_plan(n, h->fast || h->wide ? fft_elems(n, 4) : rt_elems(n, (int)h->esz));
     if (const char* inj = getenv("QG_INJECT_TMA_STALL")) h->inject_stall = atoi(inj) + 1;
     h->W = h->fast ? kFastWidth : col_width(h->plan, (int)h->esz);
@@ -1898,13 +1940,14 @@ int qg_create(const qg_grid* grid, double beta, double U, const double* mask, co
       return rc;
     }
   }
-  if (!h->fp32) {
+  {
     std::vector<double> kt(n / 2 + 1);
     for (int m = 0; m <= n / 2; ++m) kt[m] = g.kscale * m;
     void* p = nullptr;
-    if ((rc = dalloc(h, &p, kt.size() * 8)) || (rc = upload_real(h, p, kt))) { delete h; return rc; }
+    if ((rc = dalloc(h, &p, kt.size() * 8)) || (rc = upload_f64(h, p, kt))) { delete h; return rc; }
     g.kt = static_cast<const double*>(p);
   }
+  if (!h->fp32 && (rc = upload_ik2(h, &h->ik2))) { delete h; return rc; }
   // tensor maps of every mixed array for the TMA column pass
   if (h->fast) {
     const int BR = fast_box_rows(n);

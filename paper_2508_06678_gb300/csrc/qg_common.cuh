@@ -67,12 +67,13 @@ struct Geom {
   int SP;     // spectral column pitch (complex elements)
   int IP;     // mixed-array row pitch (complex elements) = Kcp
   double kscale;  // 2 pi / L
-  const double* kt;  // FP64 handles: kscale * m for m = 0 .. N / 2 (a conversion from int costs an FP64 operation)
+  float kscale_f;  // the same rounded to FP32 (FP32 passes: a conversion costs an FP64 operation)
+  const double* kt;  // kscale * m for m = 0 .. N / 2 in FP64 (a conversion from int costs an FP64 operation)
 };
 
 // wavenumber 2 pi m / L in the working precision
 template <typename T> __device__ __forceinline__ T wavenumber(const Geom& g, int m);
-template <> __device__ __forceinline__ float wavenumber<float>(const Geom& g, int m) { return float(g.kscale) * float(m); }
+template <> __device__ __forceinline__ float wavenumber<float>(const Geom& g, int m) { return g.kscale_f * float(m); }
 template <> __device__ __forceinline__ double wavenumber<double>(const Geom& g, int m) {
   const double k = __ldg(g.kt + (m < 0 ? -m : m));
   return m < 0 ? -k : k;
@@ -214,6 +215,7 @@ struct ColDesc {
   const void* visc_x;  // exp(-nu kx^2 dt), per m_x
   const void* visc_y;  // exp(-nu ky^2 dt), per r
   double visc_mu;      // exp(-mu dt)
+  const void* ik2;     // FP64 handles: 1 / |k|^2 per stored mode (NULL: divided where it is needed)
   int pdl;             // host side: launch with programmatic stream serialisation
   int lean;            // host side, FP32 Germano reduction: 0 = lean form where it makes one wave, 1 = lean form
                        // whenever it fits, 2 = never (the ensemble tuner's choice)
@@ -231,10 +233,13 @@ struct ColDesc {
 // it on the stream is still finishing: it first waits here, before any memory access, until that kernel has
 // completed and its writes are visible, then lets the next kernel be scheduled.  Launched without the
 // attribute, both instructions return at once.
+// Only what no earlier kernel of the stream writes may be read before it.
 __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+// ends the thread; every thread of the CTA takes the same decision
+__device__ __forceinline__ void leave() { asm volatile("exit;"); }
 
 // programmatic launches are allowed unless QG_NO_PDL is set in the environment (read once)
 inline bool pdl_enabled() {

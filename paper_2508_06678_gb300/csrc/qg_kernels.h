@@ -7,8 +7,9 @@ namespace qg {
 
 // Launch shape of the row pass: rows per CTA, groups (transforms side by side), physical rows kept in shared memory
 // per row (slots).
+// (the first `full` CTAs have `rows` rows, the others one)
 struct RowConfig {
-  int rows, groups, threads, nslot, one_buf, warp;
+  int full, rows, groups, threads, nslot, one_buf, warp;
   size_t smem;
 };
 RowConfig row_config(const FftPlan& p, const RowDesc& d, int esz);
@@ -16,8 +17,10 @@ template <typename T>
 cudaError_t launch_row(const Geom& g, const FftPlan& plan, const RowDesc& d, const void* tw, cudaStream_t st);
 
 // Launch shape of the column pass: w columns per CTA, fields transformed side by side, buffer pitch.
+// The first `full` CTAs do a column's work alone; each of the other columns has `split` CTAs, which all transform its
+// incoming fields and each derive a part of the outgoing ones.
 struct ColConfig {
-  int w, fields, threads, pitch, one_buf, warp;
+  int full, split, grid, w, fields, threads, pitch, one_buf, warp;
   size_t smem;
 };
 ColConfig col_config(const Geom& g, const FftPlan& p, const ColDesc& d, int W, int esz);
@@ -84,6 +87,9 @@ struct AdjCombine {
   AdjTerm term[kAdjTerms];
   double nu, mu, dt;  // AM_VISC
   int test_m2max;     // AM_TESTF
+  const double* ik2;  // 1 / |k|^2 per stored mode
+  const double *visc_x, *visc_y;  // AM_VISC, FP64 handles: exp(-nu kx^2 dt), exp(-nu ky^2 dt) (NULL: computed)
+  double visc_mu;
 };
 enum AdjKind : int { AK_NONE = 0, AK_SMAG = 1, AK_LEITH = 2 };
 enum AdjProdMode : int { AP_FORWARD = 0, AP_ADJOINT = 1 };

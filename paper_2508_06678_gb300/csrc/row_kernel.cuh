@@ -66,25 +66,26 @@ template <typename T> struct PtProducts {
 // closure 1024^2 2101 -> 1533 us, FP32 dynamic Smagorinsky 256^2 152 -> 92 us.
 template <typename T, class Sh, int PROG>
 __global__ void __launch_bounds__(pass_threads(Sh::EL, sizeof(T))) row_kernel(Geom g, Sh sh, RowConfig c, RowDesc d,
-                                                                 const cplx_t<T>* __restrict__ tw) {
-  pdl_enter();
+                                                                 const cplx_t<T>* __restrict__ twg) {
   using C = cplx_t<T>;
   constexpr int EL = Sh::EL;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int N = sh.n(), K = sh.band(g);
   const int tid = threadIdx.x, nt = blockDim.x;
   const int gi = tid / sh.tt(), t = tid - gi * sh.tt();
-  const int y0 = blockIdx.x * c.rows;
+  const int rows = (int)blockIdx.x < c.full ? c.rows : 1;
+  const int y0 = (int)blockIdx.x < c.full ? blockIdx.x * c.rows : c.full * c.rows + (blockIdx.x - c.full);
   int* const st = d.err;
   // extents for the bounds-checked debug build
   const long long n_mixed = (long long)N * g.IP, n_phys = (long long)N * N;
-  C* const bufs = reinterpret_cast<C*>(smem_raw);
+  C* const tws = reinterpret_cast<C*>(smem_raw);
+  C* const bufs = tws + (tw_shared(sh.table()) ? sh.table() : 0);
+  const C* tw = tw_stage(twg, sh.table(), tws);
+  pdl_enter();
+  const int stop = d.flag ? *reinterpret_cast<volatile int*>(d.flag) : 0;
   T* const slots = reinterpret_cast<T*>(bufs + (size_t)c.groups * (c.one_buf ? 1 : 2) * sh.buf());
   const long long nslot_el = (long long)c.rows * c.nslot * N;
   (void)n_mixed; (void)n_phys; (void)nslot_el; (void)st;
-  if (d.flag) {
-    if (__syncthreads_or(*reinterpret_cast<volatile int*>(d.flag) != 0)) return;
-  }
   FftBufs<C> fb;
   fb.active = gi < c.groups;
   fb.one = c.one_buf;
@@ -98,8 +99,8 @@ __global__ void __launch_bounds__(pass_threads(Sh::EL, sizeof(T))) row_kernel(Ge
   constexpr bool smag4 = PROG == RP_SMAG || PROG == RP_DSMAG;
   // direct programs transform item pairs that never meet: field f of row r in, the same item out
   const int nitem = direct ? (d.npair > 0 ? 2 * d.npair : d.in_phys ? d.nout : d.nin) : d.nin;
-  const int tin = row_tasks(c.rows, nitem);
-  const int tout = direct ? tin : row_tasks(c.rows, d.nout);
+  const int tin = row_tasks(rows, nitem);
+  const int tout = direct ? tin : row_tasks(rows, d.nout);
   const bool has_inv = PROG != RP_COPY || !d.in_phys, has_fwd = PROG == RP_SCALE || d.in_phys;  // of a direct program
   int bad = 0;
   C x[EL];
@@ -146,7 +147,7 @@ __global__ void __launch_bounds__(pass_threads(Sh::EL, sizeof(T))) row_kernel(Ge
     const int task = base + gi;
     const bool on = fb.active && task < (inv ? tin : tout);
     RowTask k2 = {0, 0, -1, 0};
-    if (on) k2 = row_task(task, c.rows, (inv || direct) ? nitem : d.nout);
+    if (on) k2 = row_task(task, rows, (inv || direct) ? nitem : d.nout);
     const int ya = y0 + k2.ra, yb = y0 + (k2.rb >= 0 ? k2.rb : 0);
     // an absent second field of a copy pair
     const bool two = on && k2.rb >= 0 && !(d.npair > 0 && (d.in_phys ? d.pin[k2.fb] : d.pout[k2.fb]) == nullptr);
@@ -198,6 +199,8 @@ __global__ void __launch_bounds__(pass_threads(Sh::EL, sizeof(T))) row_kernel(Ge
       }
     }
 
+    // the status flag's load has overlapped the inputs'; the barrier also completes the twiddle table
+    if (it == 0 && __syncthreads_or(stop)) return;
     sh.run(x, t, fb, tw);
 
     // ---- where the result goes
@@ -214,7 +217,7 @@ __global__ void __launch_bounds__(pass_threads(Sh::EL, sizeof(T))) row_kernel(Ge
         if (it == rin - 1) {
           __syncthreads();
           // ---- pointwise products, in place in the slots
-          const int total = c.rows * N;
+          const int total = rows * N;
           for (int e = tid; e < total; e += nt) {
             const int r = e >= N ? 1 : 0, xx = e - r * N;  // at most two rows
             T* s = slots + (size_t)r * c.nslot * N + xx;
@@ -373,7 +376,7 @@ cudaError_t launch_row_shape(const Geom& g, const FftPlan& plan, const Sh& sh, c
                              cudaStream_t st) {
   const RowConfig c = row_config(plan, d, (int)sizeof(T));
   const auto* twp = reinterpret_cast<const cplx_t<T>*>(tw);
-  const dim3 grid(g.n / c.rows), block(c.threads);
+  const dim3 grid(c.full + (g.n - c.full * c.rows)), block(c.threads);
 #define QG_ROW_P(P)                                                           \
   case P: {                                                                   \
     const cudaError_t e = raise_smem_limit<row_kernel<T, Sh, P>>(c.smem);     \
