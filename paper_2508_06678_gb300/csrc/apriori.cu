@@ -10,7 +10,7 @@
 //                   + [H F_sponge - F_sponge(H chi_s, w~)]                  (Eq. 8)
 //   model        C div(g grad w~), static (c Delta)^p or Germano/Lilly C    (Eq. 9-14)
 //   PCC          of Pi and the model over the N_c^2 points                   (Eq. 15)
-// Every transform and product runs in the generic row / column kernels of the
+// Every transform and product runs in the run-time row / column passes of the
 // time step on three grid descriptions: the fine 2/3 band, the coarse 2/3
 // band, and the coarse band without its Nyquist lines for the filtered
 // coefficient fields H chi and H chi_s (which are not truncated).
@@ -171,20 +171,62 @@ __global__ void moments_finish_kernel(const double* partials, int nblk, double* 
   }
 }
 
+// A call's device memory, zeroed: blocks of 256-byte aligned size carved from one allocation of the size reserved
+// (a hundred allocations and frees of a call took longer than its kernels), others allocated as they are asked for.
 struct Pool {
   std::vector<void*> ptrs;
   cudaError_t err = cudaSuccess;
-  void* get(size_t bytes) {
+  char* at = nullptr;
+  size_t left = 0;
+  void reserve(size_t bytes) {
+    if (err != cudaSuccess) return;
     void* p = nullptr;
-    if (err != cudaSuccess) return nullptr;
     err = cudaMalloc(&p, bytes);
-    if (err != cudaSuccess) return nullptr;
-    cudaMemset(p, 0, bytes);
+    if (err != cudaSuccess) return;
+    cudaMemsetAsync(p, 0, bytes, nullptr);
     ptrs.push_back(p);
+    at = static_cast<char*>(p);
+    left = bytes;
+  }
+  void* get(size_t bytes) {
+    const size_t need = (bytes + 255) / 256 * 256;
+    if (need > left) reserve(need);
+    if (err != cudaSuccess) return nullptr;
+    void* p = at;
+    at += need;
+    left -= need;
     return p;
   }
   ~Pool() {
     for (void* p : ptrs) cudaFree(p);
+  }
+};
+
+// Host-to-device copies beside the kernels on the legacy stream: send() starts a copy once the legacy stream has
+// reached the point of the last mark(), need() makes the legacy stream's later work wait for the last copy.
+struct Uploads {
+  cudaStream_t st = nullptr;
+  cudaEvent_t ev = nullptr;
+  cudaError_t err = cudaSuccess;
+  Uploads() {
+    err = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+    if (err == cudaSuccess) err = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+  }
+  void mark() {
+    if (err == cudaSuccess) err = cudaEventRecord(ev, nullptr);
+    if (err == cudaSuccess) err = cudaStreamWaitEvent(st, ev, 0);
+  }
+  void send(void* dst, const void* src, size_t bytes) {
+    if (err == cudaSuccess) err = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st);
+  }
+  void need() {
+    if (err == cudaSuccess) err = cudaEventRecord(ev, st);
+    if (err == cudaSuccess) err = cudaStreamWaitEvent(nullptr, ev, 0);
+  }
+  ~Uploads() {
+    if (st) cudaStreamSynchronize(st);  // the host arrays are the caller's again when the call returns
+    if (ev) cudaEventDestroy(ev);
+    if (st) cudaStreamDestroy(st);
   }
 };
 
@@ -259,6 +301,14 @@ extern "C" int qg_sgs_apriori(const double* omega_fr, int32_t n_fr, int32_t n_le
 
   Pool pool;
   Ctx cx;
+  Uploads up;
+  {
+    auto m = [](const Grid& G) { return (size_t)G.g.n * G.g.IP * 16 + 256; };
+    auto sp = [](const Grid& G) { return (size_t)G.g.Kcp * G.g.SP * 16 + 256; };
+    auto ph = [](int n) { return (size_t)n * n * 8 + 256; };
+    pool.reserve(10 * m(F) + 6 * sp(F) + 3 * ph(n_fr) + 18 * m(Cg) + m(Cf) + 14 * sp(Cg) + 2 * sp(Cf) + 7 * ph(n_les) +
+                 3 * (size_t)n_fr * 32 + (1u << 17));
+  }
   auto mixed = [&](const Grid& G) { return pool.get((size_t)G.g.n * G.g.IP * 16); };
   auto spec = [&](const Grid& G) { return pool.get((size_t)G.g.Kcp * G.g.SP * 16); };
   auto phys = [&](int n) { return pool.get((size_t)n * n * 8); };
@@ -317,9 +367,9 @@ extern "C" int qg_sgs_apriori(const double* omega_fr, int32_t n_fr, int32_t n_le
     qg::set_last_error("qg_sgs_apriori: device allocation failed");
     return QG_ERR_OOM;
   }
-  cudaMemcpy(Pw, omega_fr, nf2 * 8, cudaMemcpyHostToDevice);
-  if (mask_fr) cudaMemcpy(Pchi, mask_fr, nf2 * 8, cudaMemcpyHostToDevice);
-  if (sponge_fr) cudaMemcpy(Pchis, sponge_fr, nf2 * 8, cudaMemcpyHostToDevice);
+  up.mark();  // the memory is zeroed
+  up.send(Pw, omega_fr, nf2 * 8);
+  up.need();
 
   // test filter threshold of the coarse grid: |m|^2 (2r)^2 <= N_c^2
   int test_m2max = 0;
@@ -354,6 +404,8 @@ extern "C" int qg_sgs_apriori(const double* omega_fr, int32_t n_fr, int32_t n_le
   }
   // F_obs (unscaled): T curl(chi u); chi spectrum for its filtered coefficient field
   if (mask_fr) {
+    up.send(Pchi, mask_fr, nf2 * 8);  // while the passes above run
+    up.need();
     RowDesc r{};
     r.prog = RP_SCALE; r.nin = 2; r.nout = 2; r.in[0] = M[1]; r.in[1] = M[2]; r.out[0] = M[6]; r.out[1] = M[7];
     r.factor = Pchi;
@@ -370,6 +422,8 @@ extern "C" int qg_sgs_apriori(const double* omega_fr, int32_t n_fr, int32_t n_le
   }
   // F_sponge (unscaled): T F[chi_s w]; chi_s spectrum
   if (sponge_fr) {
+    up.send(Pchis, sponge_fr, nf2 * 8);
+    up.need();
     ColDesc c = base;
     c.op = CO_DERIVE; c.w0 = Sw; c.nder = 1; c.der[0] = D_W; c.dout[0] = M[8];
     cx.col(F, c);
@@ -521,6 +575,7 @@ extern "C" int qg_sgs_apriori(const double* omega_fr, int32_t n_fr, int32_t n_le
     moments_finish_kernel<<<1, 32, 0, cx.st>>>(mom, 256, mom + 5 * 512);
     cx.err = cudaGetLastError();
   }
+  if (cx.err == cudaSuccess) cx.err = up.err;
   if (cx.err == cudaSuccess) cx.err = cudaDeviceSynchronize();
   if (cx.err != cudaSuccess) {
     snprintf(msg, sizeof(msg), "qg_sgs_apriori: %s", cudaGetErrorString(cx.err));
