@@ -47,9 +47,13 @@ template <int N> constexpr int row_occ() {
 }
 template <int N> constexpr int col_threads();
 template <int OP, int N> struct Occ {
+  // The final passes take one CTA an SM, with more registers, where their column tiles need several rounds over the
+  // SMs either way, and two where that makes it one round (dynamic Leith 1296^2 43.5 -> 38.3 us, 1536^2 49.7 -> 42.7)
+  static constexpr int tiles = (Eng<float, N>::Kc + kFastWidth - 1) / kFastWidth;
+  static constexpr int fwd = tiles > 152 && tiles <= 304 && col_threads<N>() >= 192 ? 2 : QG_COL_MINB_FWD;
   static constexpr int want = OP == CO_DYN_REDUCE ? QG_COL_MINB_REDUCE
                               : (OP == CO_FORWARD || OP == CO_FORWARD2 || OP == CO_FORWARD_N ||
-                                 OP == CO_AB2CN_FINAL) ? QG_COL_MINB_FWD
+                                 OP == CO_AB2CN_FINAL) ? fwd
                               : OP == CO_CURL    ? QG_COL_MINB_CURL
                                                  : QG_COL_MINB;
   static constexpr int most = 512 / col_threads<N>() > 0 ? 512 / col_threads<N>() : 1;

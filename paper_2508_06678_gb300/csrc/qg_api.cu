@@ -134,7 +134,7 @@ struct qg_handle {
   void* ws = nullptr;
   void* ws2 = nullptr;  // second stage-state array (stages alternate between ws and ws2)
   void* jh = nullptr;
-  void* red_scr[3] = {nullptr, nullptr, nullptr};  // Germano reduction scratch (FP32 register-resident kernels)
+  void* red_scr[3] = {nullptr, nullptr, nullptr};  // Germano reduction scratch (FP32 fast passes)
   void* dh = nullptr;
   void* X[kMaxIn] = {};
   void* Y[kMaxY] = {};
@@ -183,7 +183,7 @@ struct qg_handle {
   int64_t step = 0;
   double t = 0;
   std::vector<void*> allocs;
-  // TMA tensor maps of the mixed arrays (power-of-two kernels)
+  // TMA tensor maps of the mixed arrays (fast passes)
   std::vector<std::pair<const void*, CUtensorMap>> maps;
   // one step captured as a CUDA graph and replayed by qg_step (eager launches
   // while tracing, or where the stream cannot be captured)
@@ -781,7 +781,7 @@ int adj_to_spec(qg_handle* h, const void* P, void* S, bool zero_mean) {
 }
 
 // spectral bands of several physical fields (at most kAdjNM): the row passes take them in pairs (one complex FFT
-// per pair; the register-resident kernels take every pair in one launch), then one column pass transforms them
+// per pair, every pair in one launch where the adjoint is fused), then one column pass transforms them
 // all, each to its own spectral array
 int adj_to_spec_many(qg_handle* h, std::initializer_list<const void*> P, std::initializer_list<void*> S) {
   std::vector<const void*> p(P);
@@ -849,7 +849,7 @@ int adj_to_phys(qg_handle* h, const void* S, std::initializer_list<int> codes, s
   int rc = run_col(h, c, QG_K_ADJ_COL, false);
   std::vector<void*> dst(P);
   if (!rc && h->adj_fused && dst.size() > 2) {
-    // every pair in one launch of the register-resident row pass
+    // every pair in one launch
     RowDesc r{};
     r.pdl = 1;
     r.prog = RP_COPY;
@@ -976,7 +976,7 @@ AdjDotOut adj_dot_out(qg_handle* h, double scale, double* out) {
   return o;
 }
 
-// Fused forms of the register-resident kernels.  Forward: the stage fields of Sw (one derive pass), one row pass
+// Fused forms.  Forward: the stage fields of Sw (one derive pass), one row pass
 // that keeps them as physical fields P[f0..] and forms J, g w_x, g w_y in registers, one column pass to the
 // spectral arrays o0 [, o1, o2].  Reverse: lam = D_W of Sl and the derivatives D_WX, D_WY of Sd (derive passes),
 // one row pass of the transposed products against the fields at P[f0..], one column pass to S[8..].
@@ -1430,7 +1430,7 @@ int adj_step(qg_handle* h) {
     if (!rc) rc = adj_combine(h, lam, false, false, {{S[8], AM_CV, 1.0}, {S[9], AM_CU, -1.0}});
   }
   if (!rc) rc = adj_combine(h, lam, false, false, {{lam, AM_VISC, 1.0}});
-  // the sponge-rate branch reads P[6], which the generic kernels' reverse stages overwrite
+  // the sponge-rate branch reads P[6], which the unfused reverse stages overwrite
   if (!rc && dotslot >= 0) rc = adj_join(h, dotslot);
   dotslot = -1;
   // the three stages in reverse: w_{s+1} = a_s w0 + b_s (w_s + dt L(w_s)); the a_s lam share of w0's gradient
@@ -1861,8 +1861,8 @@ int qg_create(const qg_grid* grid, double beta, double U, const double* mask, co
   // the passes that serve this grid
   {
     const bool generic = getenv("QG_FORCE_GENERIC") != nullptr;
-    h->fast = h->fp32 && !generic && fast_grid(n);
-    h->wide = h->fp32 && !generic && wide_grid(n);
+    h->wide = h->fp32 && !generic && wide_grid(n) && (h->dynamic || !fast_grid(n));
+    h->fast = h->fp32 && !generic && fast_grid(n) && !h->wide;
     // Programmatic launches hide the start of a step's passes behind the pass before where a pass is a few
     // microseconds and leaves SMs free; elsewhere the waiting CTAs take room from the running ones.  Measured, us per
     // step without / with: FP32 64^2 64 / 56, 192^2 102 / 95, 256^2 89 / 84, 324^2 110 / 106, 384^2 83 / 84, 512^2 120 /

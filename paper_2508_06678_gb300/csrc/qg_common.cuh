@@ -21,7 +21,7 @@
 #include <type_traits>
 #include <utility>
 
-// threads per CTA of the register-resident row pass (whole rows of N / 16 or N / 12 threads each)
+// threads per CTA of the FP32 row pass that runs a row's transforms one after another (whole groups)
 #ifndef QG_ROW_CTA_THREADS
 #define QG_ROW_CTA_THREADS 128
 #endif
@@ -118,7 +118,7 @@ enum RowProg : int {
   RP_DSMAG = 4,   // RP_SMAG at grid and test level
   RP_SCALE = 5,   // f_i * factor(x, y) for each input (Brinkman, sponge)
   RP_COPY = 6,    // identity (forward transform of a physical field, or inverse to physical)
-  // the adjoint's fused passes (register-resident kernels): the step's products of one stage with its physical
+  // the adjoint's fused passes: the step's products of one stage with its physical
   // fields kept (RP_ADJ_FWD), and the transposed products of an adjoint field with kept fields (RP_ADJ_REV)
   RP_ADJ_FWD = 7,
   RP_ADJ_REV = 8,
@@ -152,7 +152,7 @@ struct RowDesc {
   void* phys_out;
   const void* phys_in2;  // RP_COPY: a second physical field, transformed with the first (Hermitian pair)
   void* phys_out2;       // RP_COPY: the second field of an inverse pair
-  int npair;             // RP_COPY, register-resident kernels: > 0 transforms npair pairs in one launch, pair p
+  int npair;             // RP_COPY: > 0 transforms npair pairs in one launch, pair p
                          // taking physical fields pin[2p], pin[2p + 1] to out[2p], out[2p + 1] (in_phys), or
                          // mixed in[2p], in[2p + 1] to pout[2p], pout[2p + 1]; a NULL second field is skipped
   const void* pin[kMaxOut];
@@ -183,7 +183,7 @@ struct ColDesc {
   void* ws_out;    // RK stage state written when store_ws (a different array, so split passes never race)
   void* jh;        // dynamic closures: stored J_hat
   void* dh;        // dynamic closures: stored D_hat
-  void* scr[3];    // dynamic closures, FP32 register-resident kernels: the Germano reduction's cross-field
+  void* scr[3];    // dynamic closures, FP32 fast passes: the Germano reduction's cross-field
                    // values (spectral layout, kept modes only)
   int use_ws;      // the stage input is ws (else w0)
   int store_ws, store_w0;

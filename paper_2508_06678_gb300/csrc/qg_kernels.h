@@ -29,12 +29,13 @@ cudaError_t launch_col(const Geom& g, const FftPlan& plan, const ColDesc& d, con
 // columns per CTA of the column pass (the mixed arrays' pitch is a multiple of it)
 int col_width(const FftPlan& p, int esz);
 
-// FP32 grids with passes specialised for N (grid_<N>.cu): transforms side by side up to 324, one after another from
-// 384 on.  Measured around the line, us per step on an idle GPU: dynamic Smagorinsky 256^2 91 side by side and 143 one
-// after another, dynamic Leith 384^2 127 and 138, Smagorinsky 384^2 96 and 85, Leith 512^2 101 and 72.
+// FP32 grids with passes specialised for N (grid_<N>.cu): transforms side by side (wide) or one after another (fast).
+// Side by side pays while a grid leaves SMs idle and a row has enough transforms to fill them, so the dynamic closures'
+// up to 324, the others' below 192.  Measured, us per step side by side / one after another: Leith 256^2 60 / 58,
+// 324^2 108 / 94, 512^2 96 / 68; dynamic Smagorinsky 192^2 102 / 140, 256^2 89 / 105, 324^2 169 / 210, 384^2 152 / 145.
 #define QG_WIDE_GRIDS(X) X(64) X(72) X(96) X(108) X(128) X(144) X(162) X(192) X(216) X(256) X(288) X(324)
 #define QG_FAST_GRIDS(X)                                                                         \
-  X(384) X(432) X(486) X(512) X(576) X(648) X(768) X(864) X(972) X(1024) X(1152) X(1296) \
+  X(192) X(216) X(256) X(288) X(324) X(384) X(432) X(486) X(512) X(576) X(648) X(768) X(864) X(972) X(1024) X(1152) X(1296) \
   X(1458) X(1536) X(1728) X(1944) X(2048) X(2304) X(2592) X(2916) X(3072) X(3456) X(3888) X(4096)
 #define X(N) || n == N
 constexpr bool wide_grid(int n) { return false QG_WIDE_GRIDS(X); }
