@@ -137,6 +137,12 @@ template <typename C, bool PK> __device__ __forceinline__ C vsub(C a, C b) {
     return csub(a, b);
   }
 }
+// a b + c, part by part (one instruction, each part rounded as fmaf rounds it)
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)), "l"(f2_bits(c)));
+  return bits_f2(r);
+}
 // plus = t + i s d, minus = t - i s d (s = +1 / -1) with the parts of d exchanged in place
 template <typename C> __device__ __forceinline__ void rot_pm(C t, C d, int s, C& plus, C& minus) {
   if (s > 0) {
