@@ -230,24 +230,24 @@ __device__ __forceinline__ void pair_terms(const T* const (&rows)[5], int p, con
       acc2(cd[3], d, d);
       acc2(cc[3], ca_0, cb_8);
     }
-    return;
-  }
+  } else {
 #pragma unroll
-  for (int w = 0; w < W; ++w) {
-    const T a_m = x[0][w], a_0 = x[1][w], a_p = x[2][w], b_0 = x[3][w], b_8 = x[4][w];
-    const T ca_m = a_m - c[0], ca_0 = a_0 - c[1], ca_p = a_p - c[2], cb_0 = b_0 - c[3], cb_8 = b_8 - c[4];
-    T d = a_0 - b_0;
-    cd[0][w] = fma(d, d, cd[0][w]);
-    cc[0][w] = fma(ca_0, cb_0, cc[0][w]);
-    d = a_m - b_0;
-    cd[1][w] = fma(d, d, cd[1][w]);
-    cc[1][w] = fma(ca_m, cb_0, cc[1][w]);
-    d = a_p - b_8;
-    cd[2][w] = fma(d, d, cd[2][w]);
-    cc[2][w] = fma(ca_p, cb_8, cc[2][w]);
-    d = a_0 - b_8;
-    cd[3][w] = fma(d, d, cd[3][w]);
-    cc[3][w] = fma(ca_0, cb_8, cc[3][w]);
+    for (int w = 0; w < W; ++w) {
+      const T a_m = x[0][w], a_0 = x[1][w], a_p = x[2][w], b_0 = x[3][w], b_8 = x[4][w];
+      const T ca_m = a_m - c[0], ca_0 = a_0 - c[1], ca_p = a_p - c[2], cb_0 = b_0 - c[3], cb_8 = b_8 - c[4];
+      T d = a_0 - b_0;
+      cd[0][w] = fma(d, d, cd[0][w]);
+      cc[0][w] = fma(ca_0, cb_0, cc[0][w]);
+      d = a_m - b_0;
+      cd[1][w] = fma(d, d, cd[1][w]);
+      cc[1][w] = fma(ca_m, cb_0, cc[1][w]);
+      d = a_p - b_8;
+      cd[2][w] = fma(d, d, cd[2][w]);
+      cc[2][w] = fma(ca_p, cb_8, cc[2][w]);
+      d = a_0 - b_8;
+      cd[3][w] = fma(d, d, cd[3][w]);
+      cc[3][w] = fma(ca_0, cb_8, cc[3][w]);
+    }
   }
 }
 
