@@ -61,27 +61,6 @@ void make_grid(Grid& G, int n, int K, double L, int nslot) {
   G.row_smem = (size_t)n * 16 + (size_t)(nslot > 2 ? nslot : 2) * n * 8;
 }
 
-void cos_sin_frac(long j, long n, double* c, double* s) {
-  j %= n;
-  const long q4 = 4 * j, quad = q4 / n, rem = q4 - quad * n;
-  double cc, ss;
-  if (2 * rem <= n) {
-    const double phi = (M_PI / 2) * double(rem) / double(n);
-    cc = std::cos(phi);
-    ss = std::sin(phi);
-  } else {
-    const double phi = (M_PI / 2) * double(n - rem) / double(n);
-    cc = std::sin(phi);
-    ss = std::cos(phi);
-  }
-  switch (quad) {
-    case 0: *c = cc; *s = ss; break;
-    case 1: *c = -ss; *s = cc; break;
-    case 2: *c = -cc; *s = -ss; break;
-    default: *c = ss; *s = -cc; break;
-  }
-}
-
 // Eq. 5: out(m) = scale * H(m) * in(m) on the output grid's stored modes,
 // H = exp(-k^2 Delta^2 / 6) (optional) times the cut-off |m| <= N_c / 2.
 __global__ void filter_copy_kernel(Geom gi, const C2* __restrict__ in, Geom go, C2* __restrict__ out, int n_c,
@@ -314,13 +293,7 @@ extern "C" int qg_sgs_apriori(const double* omega_fr, int32_t n_fr, int32_t n_le
   auto phys = [&](int n) { return pool.get((size_t)n * n * 8); };
   // twiddles per grid size
   for (Grid* G : {&F, &Cg, &Cf}) {
-    std::vector<double> tw(2 * (size_t)G->plan.table);
-    for (int e = 0; e < G->plan.table; ++e) {
-      double c, s;
-      cos_sin_frac(fft_table_exponent(G->plan, e), G->g.n, &c, &s);
-      tw[2 * e] = c;
-      tw[2 * e + 1] = -s;
-    }
+    std::vector<double> tw = fft_table(G->plan, 8);
     // twiddles, then the wavenumbers 2 pi m / L
     for (int m = 0; m <= G->g.n / 2; ++m) tw.push_back(G->g.kscale * m);
     G->tw = pool.get(tw.size() * 8);
@@ -645,13 +618,7 @@ extern "C" int qg_grid_filter(const double* omega_fr, int32_t nsnap, int32_t n_f
   Pool pool;
   Ctx cx;
   for (Grid* G : {&F, &Cg}) {
-    std::vector<double> tw(2 * (size_t)G->plan.table);
-    for (int e = 0; e < G->plan.table; ++e) {
-      double c, s;
-      cos_sin_frac(fft_table_exponent(G->plan, e), G->g.n, &c, &s);
-      tw[2 * e] = c;
-      tw[2 * e + 1] = -s;
-    }
+    std::vector<double> tw = fft_table(G->plan, 8);
     // twiddles, then the wavenumbers 2 pi m / L
     for (int m = 0; m <= G->g.n / 2; ++m) tw.push_back(G->g.kscale * m);
     G->tw = pool.get(tw.size() * 8);

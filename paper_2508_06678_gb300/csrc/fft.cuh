@@ -19,6 +19,8 @@
 // loaded and stored one by one.
 #pragma once
 
+#include <vector>
+
 #include "qg_common.cuh"
 
 namespace qg {
@@ -86,16 +88,26 @@ struct FftPlan {
 
 // plan for n = 2^a 3^b (even, 16..4096) with el elements per thread
 FftPlan fft_plan(int n, int el);
-// entry e of the plan's twiddle table is exp(-2 pi i j / n) with this j = r k n / (ns R)
-__host__ __device__ inline int fft_table_exponent(const FftPlan& p, int e) {
+// Entry e of the plan's twiddle table belongs to a pass of this radix and stands for w = exp(-2 pi i j / n) with this
+// j = r k n / (ns R).
+struct FftEntry {
+  int j, radix;
+};
+__host__ __device__ inline FftEntry fft_table_entry(const FftPlan& p, int e) {
   for (int i = p.npass - 1; i >= 1; --i) {
     const FftPass& s = p.pass[i];
     if (e < s.off) continue;
     const int r = (e - s.off) / s.ns + 1, k = (e - s.off) % s.ns;
-    return (int)(((long long)r * k * (p.n / (s.ns * s.radix))) % p.n);
+    return {(int)(((long long)r * k * (p.n / (s.ns * s.radix))) % p.n), s.radix};
   }
-  return 0;
+  return {0, 0};
 }
+// FP64 passes of radix 2 and 4 take a twiddle w = c + i s as (c, s / c) (see twiddled), others as (c, s)
+__host__ __device__ constexpr bool ratio_twiddle(int radix, int esz) { return esz == 8 && (radix == 2 || radix == 4); }
+// for w = +-i, c is this instead of 0: c (s / c) is s still, and c itself, 1e-18, is nothing beside it
+constexpr double kRatioMinCos = 1.0 / (1ll << 60);
+// the table of the plan for elements of esz bytes (plan.cu): pairs of doubles, each the rounding of its exact value
+std::vector<double> fft_table(const FftPlan& p, int esz);
 
 template <typename C> __device__ __forceinline__ C cmulk(C a, decltype(C::x) c, decltype(C::x) s) {
   return mk<C>(a.x * c - a.y * s, a.x * s + a.y * c);
@@ -371,16 +383,22 @@ template <typename C> struct FftBufs {
   }
 };
 
-// (a, b) <- (a + w b, a - w b): the difference is 2 a minus the sum
-template <typename C> __device__ __forceinline__ void bfly(C& a, C& b, C w) {
-  using T = decltype(C::x);
-  const T sx = fma(-w.y, b.y, fma(w.x, b.x, a.x)), sy = fma(w.y, b.x, fma(w.x, b.y, a.y));
-  b = mk<C>(fma(T(2), a.x, -sx), fma(T(2), a.y, -sy));
-  a = mk<C>(sx, sy);
+// b (1 + i q) = b w / c for the twiddle w = c (1 + i q), given as (c, q)
+template <typename C> __device__ __forceinline__ C tw_turn(C b, C w) {
+  return mk<C>(fma(-w.y, b.y, b.x), fma(w.y, b.x, b.y));
+}
+// (a, b) <- (a + c b, a - c b)
+template <typename C> __device__ __forceinline__ void tw_sums(C& a, C& b, decltype(C::x) c) {
+  const C s = mk<C>(fma(c, b.x, a.x), fma(c, b.y, a.y));
+  b = mk<C>(fma(-c, b.x, a.x), fma(-c, b.y, a.y));
+  a = s;
 }
 // Butterfly of radix R with its twiddles w[(r - 1) ns] (kernel exp(s 2 pi i / N): conjugated for s > 0).  FP64 radices
-// 2 and 4 fuse the twiddles into the butterflies (w v1 + w^3 v3 = w (v1 + w^2 v3)): six FMA-pipe operations per
-// two-point butterfly against eight, and two twiddle loads for radix 4 against three.
+// 2 and 4 take them as cosine and tangent, the cosine joining the first sums (Linzer and Feig, "Implementation of
+// efficient FFT algorithms on fused multiply-add architectures", 1993): six operations for radix 2 against eight, 24
+// for radix 4 against 28.  Every element meets one table entry and every sum rounds once.  Forming a difference as
+// 2 a minus the sum, and v3's twiddle as a product of two entries, takes 24 operations too, but adds the sum's and
+// the second entry's roundings.
 // GL: the table lies in global memory (else in shared memory or anywhere).
 template <bool GL, typename C> __device__ __forceinline__ C tw_load(const C* w) {
   if constexpr (GL) return __ldg(w);
@@ -389,21 +407,24 @@ template <bool GL, typename C> __device__ __forceinline__ C tw_load(const C* w) 
 template <typename C, int R, bool PK, bool GL>
 __device__ __forceinline__ void twiddled(C* v, const C* w, int ns, int s) {
   using T = decltype(C::x);
-  if constexpr (sizeof(T) == 8 && (R == 2 || R == 4)) {
+  if constexpr (ratio_twiddle(R, sizeof(T))) {
     C w1 = tw_load<GL>(w);
     if (s > 0) w1.y = -w1.y;
+    v[1] = tw_turn(v[1], w1);
     if constexpr (R == 2) {
-      bfly(v[0], v[1], w1);
+      tw_sums(v[0], v[1], w1.x);
     } else {
-      C w2 = tw_load<GL>(w + ns);
-      if (s > 0) w2.y = -w2.y;
-      bfly(v[0], v[2], w2);
-      bfly(v[1], v[3], w2);
-      bfly(v[0], v[1], w1);
-      bfly(v[2], v[3], cmul_si(w1, s));
-      const C o2 = v[1];
-      v[1] = v[2];
-      v[2] = o2;
+      C w2 = tw_load<GL>(w + ns), w3 = tw_load<GL>(w + 2 * ns);
+      if (s > 0) {
+        w2.y = -w2.y;
+        w3.y = -w3.y;
+      }
+      C a = v[0], b = tw_turn(v[2], w2), c = cscale(v[1], w1.x), d = tw_turn(v[3], w3);
+      tw_sums(a, b, w2.x);
+      tw_sums(c, d, w3.x);
+      v[0] = cadd(a, c);
+      v[2] = csub(a, c);
+      rot_pm(b, d, s, v[1], v[3]);
     }
   } else {
 #pragma unroll

@@ -60,8 +60,13 @@ template <typename T>
 __global__ void twiddle_kernel(cplx_t<T>* tw, FftPlan plan, double* kt, double kscale) {
   for (int m = blockIdx.x * blockDim.x + threadIdx.x; m <= plan.n / 2; m += gridDim.x * blockDim.x) kt[m] = kscale * m;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < plan.table; e += gridDim.x * blockDim.x) {
+    const FftEntry f = fft_table_entry(plan, e);
     double s, c;
-    sincospi(2.0 * double(fft_table_exponent(plan, e)) / double(plan.n), &s, &c);
+    sincospi(2.0 * double(f.j) / double(plan.n), &s, &c);
+    if (ratio_twiddle(f.radix, sizeof(T))) {
+      if (fabs(c) < kRatioMinCos) c = kRatioMinCos;
+      s /= c;
+    }
     tw[e] = mk<cplx_t<T>>(T(c), T(-s));
   }
 }

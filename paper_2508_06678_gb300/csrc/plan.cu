@@ -1,6 +1,9 @@
 // Host side of the run-time FFT engine (fft.cuh): plans, and the launch shapes of the passes that use it.
 #include "qg_kernels.h"
 
+#include <cmath>
+#include <utility>
+
 namespace qg {
 
 FftPlan fft_plan(int n, int el) {
@@ -15,6 +18,72 @@ FftPlan fft_plan(int n, int el) {
   p.table = r.table;
   p.buf = n + n / 16 + 1;
   return p;
+}
+
+// ---- twiddle tables.  A table's rounding errors are the same in every transform, so they add up from step to step;
+// the entries are formed in double-double arithmetic (a value as the unevaluated sum h + l) and rounded once.
+namespace {
+struct DD {
+  double h, l;
+};
+DD norm(double a, double b) {  // |a| >= |b|
+  const double s = a + b;
+  return {s, b - (s - a)};
+}
+DD add(DD a, DD b) {
+  const double s = a.h + b.h, t = s - a.h;
+  return norm(s, (a.h - (s - t)) + (b.h - t) + (a.l + b.l));
+}
+DD neg(DD a) { return {-a.h, -a.l}; }
+DD mul(DD a, DD b) {
+  const double p = a.h * b.h;
+  return norm(p, std::fma(a.h, b.h, -p) + std::fma(a.h, b.l, a.l * b.h));
+}
+DD div(DD a, double b) {
+  const double q = a.h / b;
+  return norm(q, (std::fma(-q, b, a.h) + a.l) / b);
+}
+struct Rot {
+  DD c, s;
+};
+Rot turn(const Rot& a, const Rot& b) {
+  return {add(mul(a.c, b.c), neg(mul(a.s, b.s))), add(mul(a.s, b.c), mul(a.c, b.s))};
+}
+}  // namespace
+
+std::vector<double> fft_table(const FftPlan& p, int esz) {
+  // cos and sin of 2 pi i / (4 n) for angles up to pi / 4: the smallest by its Taylor series, the others by addition
+  const long n = p.n;
+  std::vector<Rot> rot(n / 2 + 1);
+  rot[0] = {{1.0, 0.0}, {0.0, 0.0}};
+  const DD x = div(DD{1.5707963267948966, 6.123233995736766e-17}, (double)n);
+  Rot r = rot[0];
+  DD term = {1.0, 0.0};
+  for (int k = 1; k < 24; ++k) {
+    term = div(mul(term, x), k);
+    DD& sum = k & 1 ? r.s : r.c;
+    sum = add(sum, k & 2 ? neg(term) : term);
+  }
+  rot[1] = r;
+  for (long i = 2; i <= n / 2; ++i) rot[i] = turn(rot[i / 2], rot[i - i / 2]);
+  std::vector<double> t(2 * (size_t)p.table);
+  for (int e = 0; e < p.table; ++e) {
+    const FftEntry f = fft_table_entry(p, e);
+    const long q4 = 4L * f.j, quad = q4 / n, rem = q4 - quad * n;  // the angle within its quadrant is (pi / 2) rem / n
+    const bool low = 2 * rem <= n;
+    const Rot& w = rot[low ? rem : n - rem];
+    DD c = low ? w.c : w.s, s = low ? w.s : w.c;
+    if (quad & 1) std::swap(c, s);
+    if (quad == 1 || quad == 2) c = neg(c);
+    if (quad < 2) s = neg(s);  // exp(-i angle)
+    t[2 * e] = c.h;
+    t[2 * e + 1] = s.h;
+    if (ratio_twiddle(f.radix, esz)) {
+      if (std::fabs(c.h) < kRatioMinCos) t[2 * e] = kRatioMinCos;
+      t[2 * e + 1] = div(s, t[2 * e]).h;
+    }
+  }
+  return t;
 }
 
 // dynamic shared memory a CTA can have: 227 KB less the passes' static part (under 768 bytes)

@@ -73,31 +73,6 @@ bool valid_n(int n) {
   return m == 1;
 }
 
-// cos and sin of 2 pi j / n with the argument reduced exactly to [0, pi/4].
-void cos_sin_frac(long j, long n, double* c, double* s) {
-  j %= n;
-  if (j < 0) j += n;
-  const long q4 = 4 * j;
-  const long quad = q4 / n;
-  const long rem = q4 - quad * n;  // angle within the quadrant = (pi/2) rem / n
-  double cc, ss;
-  if (2 * rem <= n) {
-    const double phi = (M_PI / 2) * double(rem) / double(n);
-    cc = std::cos(phi);
-    ss = std::sin(phi);
-  } else {
-    const double phi = (M_PI / 2) * double(n - rem) / double(n);
-    cc = std::sin(phi);
-    ss = std::cos(phi);
-  }
-  switch (quad) {
-    case 0: *c = cc; *s = ss; break;
-    case 1: *c = -ss; *s = cc; break;
-    case 2: *c = -cc; *s = -ss; break;
-    default: *c = ss; *s = -cc; break;
-  }
-}
-
 }  // namespace
 
 namespace qg {
@@ -1922,19 +1897,7 @@ int qg_create(const qg_grid* grid, double beta, double U, const double* mask, co
 
   // twiddles exp(-2 pi i j / n)
   {
-    std::vector<double> tw(2 * (size_t)n);
-    for (int j = 0; j < n; ++j) {
-      double c, s;
-      cos_sin_frac(j, n, &c, &s);
-      tw[2 * j] = c;
-      tw[2 * j + 1] = -s;
-    }
-    std::vector<double> pt(2 * (size_t)h->plan.table);
-    for (int e = 0; e < h->plan.table; ++e) {
-      const int j = fft_table_exponent(h->plan, e);
-      pt[2 * e] = tw[2 * j];
-      pt[2 * e + 1] = tw[2 * j + 1];
-    }
+    const std::vector<double> pt = fft_table(h->plan, (int)h->esz);
     if ((rc = dalloc(h, &h->ptw, pt.size() / 2 * csz)) || (rc = upload_real(h, h->ptw, pt))) {
       delete h;
       return rc;
