@@ -348,7 +348,10 @@ __global__ void __launch_bounds__(pass_threads(Sh::EL, sizeof(T))) col_kernel(Ge
             }
           }
           if (nder > 0) {
-            wn = cscale(wn, scale);
+            if constexpr (sizeof(T) == 8 && EL % 3 == 0)  // N has factors of 3
+              wn = mk<C>(fma(wn.x, scale, wn.x * cs.scale_lo), fma(wn.y, scale, wn.y * cs.scale_lo));
+            else
+              wn = cscale(wn, scale);
             QG_ST(slotA, e, nspec, st, wn);
             QG_ST(slotB, e, nspec, st, mk<C>(-wn.x * ik2, -wn.y * ik2));
           }

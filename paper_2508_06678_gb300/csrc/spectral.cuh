@@ -7,6 +7,8 @@
 // all warps of a CTA add up the partial sums where one warp did.
 #pragma once
 
+#include <cmath>
+
 #include "qg_kernels.h"
 
 namespace qg {
@@ -14,6 +16,7 @@ namespace qg {
 constexpr int kIk2Small = 16;  // FP32: 1 / |k|^2 up to this |m|^2 is inverted in FP64 before rounding
 template <typename T> struct ColScalars {
   T ks, ks2, dt, a, b, beta, U, coeff, rpow, inv_eta, nu, mu, visc_mu, scale;
+  T scale_lo;  // FP64: 1 / N^2 less its rounding (the same sign in every step), 0 for N = 2^a
   T ik2s[kIk2Small + 1];
 };
 template <typename T> ColScalars<T> col_scalars(const Geom& g, const ColDesc& d) {
@@ -32,7 +35,9 @@ template <typename T> ColScalars<T> col_scalars(const Geom& g, const ColDesc& d)
   s.nu = T(d.nu);
   s.mu = T(d.mu);
   s.visc_mu = T(d.visc_mu);
-  s.scale = T(1.0 / (double(g.n) * double(g.n)));
+  const double n2 = double(g.n) * double(g.n), inv = 1.0 / n2;
+  s.scale = T(inv);
+  s.scale_lo = sizeof(T) == 8 ? T(-std::fma(inv, n2, -1.0) * inv) : T(0);
   s.ik2s[0] = T(0);
   for (int m = 1; m <= kIk2Small; ++m) s.ik2s[m] = T(1.0 / (ks2 * double(m)));
   return s;

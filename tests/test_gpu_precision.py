@@ -7,7 +7,8 @@ errors that are the same in every step (of the twiddle tables, of 1 / N^2, of th
 
 The bounds are 1.1 times (the spread from one set of fields to another) what plain Stockham transforms of radix 8 or 16,
 4, 2 and 3 with the twiddles multiplied one by one gave in the same runs on a GB300: 7.37e-15 at 128^2, 1.18e-14 at
-256^2, 2.07e-14 at 512^2, 4.48e-14 at 1024^2.
+256^2, 2.07e-14 at 512^2, 4.48e-14 at 1024^2; 8.42e-15 at 72^2, 7.58e-15 at 96^2, 1.48e-14 at 108^2, 1.20e-14 at 144^2,
+1.32e-14 at 192^2, 1.77e-14 at 216^2, 1.97e-14 at 384^2, 4.51e-14 at 768^2.
 """
 import numpy as np
 import pytest
@@ -53,4 +54,13 @@ POWERS_OF_TWO = [(128, 20, 8.1e-15), (256, 20, 1.3e-14), (512, 10, 2.3e-14), (10
 
 @pytest.mark.parametrize("n,steps,bound", POWERS_OF_TWO)
 def test_round_trips_of_the_state_powers_of_two(n, steps, bound):
+    assert round_trip_error(n, steps) < bound
+
+
+FACTORS_OF_THREE = [(72, 20, 9.3e-15), (96, 20, 8.3e-15), (108, 20, 1.63e-14), (144, 20, 1.32e-14), (192, 20, 1.45e-14),
+                    (216, 20, 1.95e-14), (384, 10, 2.17e-14), (768, 10, 4.96e-14)]
+
+
+@pytest.mark.parametrize("n,steps,bound", FACTORS_OF_THREE)
+def test_round_trips_of_the_state_factors_of_three(n, steps, bound):
     assert round_trip_error(n, steps) < bound
