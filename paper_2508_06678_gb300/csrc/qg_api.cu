@@ -94,7 +94,7 @@ struct qg_handle {
   // the passes that serve the grid: run-time transforms (FP64, and the smallest FP32 grids), or passes specialised
   // for N that run a row's or column's transforms side by side (wide), or one after another with TMA tiles (fast)
   bool wide = false, fast = false;
-  bool adj_fused = false;  // the adjoint's fused row passes fit in shared memory
+  bool adj_fused = false;  // the adjoint's products are formed in its row passes
   bool dynamic = false;
   double static_coeff = 0.0;
   int test_m2max = 0;  // largest |m|^2 the test filter keeps
@@ -663,13 +663,12 @@ constexpr int kAdjNM = 8;   // mixed: the outputs of one derive pass, or one bat
 constexpr int kAdjStageP = 19;  // first of the per-stage physical fields (u, v, w_x, w_y, psi_xy, psi_d)
 constexpr int kAdjStageS = 19;  // first of the per-stage spectral SGS fluxes F[g w_x], F[g w_y]
 // dynamic closures only: per stage the test-level state G w, H and M (spectral), G w's fields (physical),
-// scratch spectra, one physical scratch field, and four device scalars <HM>, <MM>, C, kappa per stage
+// scratch spectra, and four device scalars <HM>, <MM>, C, kappa per stage
 constexpr int kAdjDynS = 25;       // 3 x (G w, H, M)
 constexpr int kAdjDynTmpS = 34;    // 5 scratch spectra
 constexpr int kAdjNSDyn = 39;
 constexpr int kAdjDynP = 37;       // 3 x 6 fields of G w
-constexpr int kAdjDynMuP = 55;     // the field mu = M (or G M)
-constexpr int kAdjNPDyn = 56;
+constexpr int kAdjNPDyn = 55;
 constexpr int kAdjScalars = 8;     // offset of the per-stage scalars after the dot results
 
 int adj_alloc(qg_handle* h) {
@@ -916,7 +915,7 @@ int adj_stage_fields(qg_handle* h, const void* Sw, int kind, int f0) {
   return adj_to_phys(h, Sw, {D_U, D_V, D_WX, D_WY}, {P[f0], P[f0 + 1], P[f0 + 2], P[f0 + 3]});
 }
 
-AdjProducts adj_prod_desc(qg_handle* h, int kind, int mode, int f0, int lam = 6) {
+AdjProducts adj_prod_desc(qg_handle* h, int kind, int mode, int f0) {
   auto& P = h->adj_P;
   AdjProducts a{};
   a.kind = kind;
@@ -927,7 +926,7 @@ AdjProducts adj_prod_desc(qg_handle* h, int kind, int mode, int f0, int lam = 6)
   a.wy = P[f0 + 3];
   a.pxy = P[f0 + 4];
   a.pd = P[f0 + 5];
-  a.lam = P[lam];
+  a.lam = P[6];
   a.lx = P[7];
   a.ly = P[8];
   for (int k = 0; k < 8; ++k) a.out[k] = P[9 + k];
@@ -1058,7 +1057,6 @@ int adj_fused_rev_tail(qg_handle* h, int kind, int f0) {
 // SJ holds J(w); the stage's SGS flux spectra hold F[g w_x], F[g w_y].
 int adj_forward_germano(qg_handle* h, int kind, const void* Sw, const void* SJ, int s) {
   auto& S = h->adj_S;
-  auto& P = h->adj_P;
   void* Swt = S[kAdjDynS + 3 * s];
   void* SH = S[kAdjDynS + 3 * s + 1];
   void* SM = S[kAdjDynS + 3 * s + 2];
@@ -1071,13 +1069,7 @@ int adj_forward_germano(qg_handle* h, int kind, const void* Sw, const void* SJ, 
   const double rp = std::pow(h->cl.test_ratio, kind == AK_SMAG ? 2 : 3);
   const double n4 = std::pow(double(h->g.n), 4);
   int rc = adj_combine(h, Swt, false, false, {{Sw, AM_ONE | AM_TESTF, 1.0}});
-  if (h->adj_fused) {
-    if (!rc) rc = adj_fused_fwd(h, kind, Swt, f0, T0, T1, T2);
-  } else {
-    if (!rc) rc = adj_stage_fields(h, Swt, kind, f0);
-    if (!rc) rc = adj_products(h, adj_prod_desc(h, kind, AP_FORWARD, f0));
-    if (!rc) rc = adj_to_spec_many(h, {P[9], P[10], P[11]}, {T0, T1, T2});
-  }
+  if (!rc) rc = adj_fused_fwd(h, kind, Swt, f0, T0, T1, T2);
   if (!rc) rc = adj_combine(h, SH, false, false, {{T0, AM_ONE, 1.0}, {SJ, AM_ONE | AM_TESTF, -1.0}});
   if (!rc)
     rc = adj_combine(h, SM, false, false,
@@ -1126,7 +1118,6 @@ int adj_forward_stage(qg_handle* h, int kind, bool dyn, double C, const void* S0
 //   kappa [G J'(G w)^T M - J'(w)^T G M + r^p G D'(G w)^T nu - D'(w)^T G nu],  nu = H - 2 C M
 int adj_reverse_germano(qg_handle* h, int kind, void* Slam_out, int s) {
   auto& S = h->adj_S;
-  auto& P = h->adj_P;
   const void* SH = S[kAdjDynS + 3 * s + 1];
   const void* SM = S[kAdjDynS + 3 * s + 2];
   void* Snu = S[kAdjDynTmpS + 3];
@@ -1134,41 +1125,19 @@ int adj_reverse_germano(qg_handle* h, int kind, void* Slam_out, int s) {
   const double* C = adj_scalar(h, s, 2);
   double* kappa = adj_scalar(h, s, 3);  // set by the stage's C-derivative dot (adj_reverse_stage)
   const double rp = std::pow(h->cl.test_ratio, kind == AK_SMAG ? 2 : 3);
-  const int mu = kAdjDynMuP;
   int rc = adj_combine(h, Snu, false, false, {{SH, AM_ONE, 1.0}, {SM, AM_ONE, -2.0, C}});
   // outer group, at the test-level state, filtered afterwards: mu = M, derivatives of nu
-  if (h->adj_fused) {
-    if (!rc) rc = adj_derive(h, SM, {D_W}, 0);
-    if (!rc) rc = adj_derive(h, Snu, {D_WX, D_WY}, 1);
-  } else {
-    if (!rc) rc = adj_to_phys(h, SM, {D_W}, {P[mu]});
-    if (!rc) rc = adj_to_phys(h, Snu, {D_WX, D_WY}, {P[7], P[8]});
-    if (!rc) rc = adj_products(h, adj_prod_desc(h, kind, AP_ADJOINT, kAdjDynP + 6 * s, mu));
-  }
+  if (!rc) rc = adj_derive(h, SM, {D_W}, 0);
+  if (!rc) rc = adj_derive(h, Snu, {D_WX, D_WY}, 1);
   for (int pass = 0; pass < 2 && !rc; ++pass) {
     if (pass == 1) {
       // inner group, at the stage state: mu = G M, derivatives of G nu
       rc = adj_combine(h, Sg, false, false, {{SM, AM_ONE | AM_TESTF, 1.0}});
-      if (h->adj_fused) {
-        if (!rc) rc = adj_derive(h, Sg, {D_W}, 0);
-      } else {
-        if (!rc) rc = adj_to_phys(h, Sg, {D_W}, {P[mu]});
-      }
+      if (!rc) rc = adj_derive(h, Sg, {D_W}, 0);
       if (!rc) rc = adj_combine(h, Sg, false, false, {{Snu, AM_ONE | AM_TESTF, 1.0}});
-      if (h->adj_fused) {
-        if (!rc) rc = adj_derive(h, Sg, {D_WX, D_WY}, 1);
-      } else {
-        if (!rc) rc = adj_to_phys(h, Sg, {D_WX, D_WY}, {P[7], P[8]});
-        if (!rc) rc = adj_products(h, adj_prod_desc(h, kind, AP_ADJOINT, kAdjStageP + 6 * s, mu));
-      }
+      if (!rc) rc = adj_derive(h, Sg, {D_WX, D_WY}, 1);
     }
-    if (!rc && h->adj_fused)
-      rc = adj_fused_rev_tail(h, kind, pass == 0 ? kAdjDynP + 6 * s : kAdjStageP + 6 * s);
-    else if (!rc && kind == AK_SMAG)
-      rc = adj_to_spec_many(h, {P[9], P[10], P[11], P[12], P[13], P[14], P[15], P[16]},
-                            {S[8], S[9], S[10], S[11], S[12], S[13], S[14], S[15]});
-    else if (!rc)
-      rc = adj_to_spec_many(h, {P[9], P[10], P[11], P[12], P[13], P[14]}, {S[8], S[9], S[10], S[11], S[12], S[13]});
+    if (!rc) rc = adj_fused_rev_tail(h, kind, pass == 0 ? kAdjDynP + 6 * s : kAdjStageP + 6 * s);
     if (rc) return rc;
     const int f = pass == 0 ? AM_TESTF : 0;
     const double sj = pass == 0 ? 1.0 : -1.0, sd = pass == 0 ? rp : -1.0;
@@ -1848,7 +1817,10 @@ int qg_create(const qg_grid* grid, double beta, double U, const double* mask, co
     if (const char* inj = getenv("QG_INJECT_TMA_STALL")) h->inject_stall = atoi(inj) + 1;
     h->W = h->fast ? kFastWidth : col_width(h->plan, (int)h->esz);
     const size_t adj_slots = closure->kind == QG_NONE ? 4 : closure->kind == QG_LEITH || closure->kind == QG_DLEITH ? 6 : 8;
-    h->adj_fused = h->fast || adj_slots * n * h->esz + h->plan.buf * csz <= smem_cap;
+    // The dynamic closures' always fit: the step's own row pass keeps eight or twelve rows.  The static ones' do not for
+    // FP64 Smagorinsky from 2916 and Leith from 3888, which take the products' passes apart; so does any grid under
+    // QG_FORCE_GENERIC, where those passes can be checked on small ones.
+    h->adj_fused = h->fast || h->dynamic || (!generic && adj_slots * n * h->esz + h->plan.buf * csz <= smem_cap);
   }
   g.Kcp = (g.Kc + h->W - 1) / h->W * h->W;
   g.IP = g.Kcp;
