@@ -20,7 +20,6 @@
 #include "fft.cuh"
 #include "qg_kernels.h"
 #include "spectral.cuh"
-#include "tma.cuh"
 
 namespace qg {
 
@@ -61,19 +60,6 @@ __global__ void __launch_bounds__(pass_threads(Sh::EL, sizeof(T))) col_kernel(Ge
   const long long n_mixed = (long long)N * g.IP, n_spec = (long long)g.Kcp * g.SP;
   const long long n_part = 2LL * gridDim.x;  // Germano partial sums: two per column CTA
   (void)n_mixed; (void)n_spec; (void)n_part; (void)st;
-
-
-  if (d.stall_cta1 == (int)blockIdx.x + 1 && d.nfwd > 0) {
-    // injected stall (failure-handling test): a wait for a tile that is never requested runs out after its bound
-    __shared__ __align__(8) uint64_t bar;
-    if (tid == 0) {
-      tma::mbar_init(&bar, 1);
-      tma::fence_mbar_init();
-      tma::mbar_expect_tx(&bar, 16);
-      if (!tma::mbar_wait(&bar, 0, tma::kWaitCycles) && d.err) atomicOr(d.err, kFlagTimeout);
-    }
-    return;
-  }
 
   // this thread's group: field slot fl, column c, position t
   const int fl = tid / (sh.tt() * W);

@@ -6,6 +6,7 @@
 // two-level and deterministic: fixed per-block partials, then one block sums
 // them in a fixed order.
 #include "qg_kernels.h"
+#include "tma.cuh"
 
 namespace qg {
 
@@ -135,6 +136,20 @@ template <typename S, typename D>
 __global__ void convert_kernel(const S* __restrict__ src, D* __restrict__ dst, size_t count) {
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x)
     dst[i] = D(src[i]);
+}
+
+// Failure-handling test, for handles whose column passes wait for no tile: a wait that runs out after its bound and
+// raises the status bit, before the first of them.
+__global__ void stall_kernel(int* err) {
+  __shared__ __align__(8) uint64_t bar;
+  tma::mbar_init(&bar, 1);
+  tma::fence_mbar_init();
+  tma::mbar_expect_tx(&bar, 16);  // of a copy that is never requested
+  if (!tma::mbar_wait(&bar, 0, tma::kWaitCycles)) atomicOr(err, kFlagTimeout);
+}
+cudaError_t launch_stall(int* err, cudaStream_t st) {
+  stall_kernel<<<1, 1, 0, st>>>(err);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_convert(const void* src, int src_fp32, void* dst, int dst_fp32, size_t count, cudaStream_t st) {

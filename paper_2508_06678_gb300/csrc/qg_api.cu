@@ -434,6 +434,16 @@ void set_after_rk(qg_handle* h, ColDesc& d) {
   }
 }
 
+// the injected stall (QG_INJECT_TMA_STALL) goes to the first column pass with inputs: a tile that one of its CTAs never
+// requests, or a wait in front of it where the passes have no tiles to wait for
+int take_stall(qg_handle* h, ColDesc& c) {
+  const int stall = h->inject_stall;
+  h->inject_stall = 0;
+  if (h->fast) c.stall_cta1 = stall;
+  else if (stall) CK(launch_stall(h->flag, h->stream), "injected stall");
+  return QG_OK;
+}
+
 const double kRK[3][2] = {{0.0, 1.0}, {0.75, 0.25}, {1.0 / 3.0, 2.0 / 3.0}};
 
 int enqueue_step(qg_handle* h) {
@@ -460,8 +470,7 @@ int enqueue_step(qg_handle* h) {
       cr.op = CO_DYN_REDUCE;
       cr.nfwd = 6;
       for (int i = 0; i < 6; ++i) cr.fin[i] = h->Y[i];
-      cr.stall_cta1 = h->inject_stall;
-      h->inject_stall = 0;
+      if ((rc = take_stall(h, cr))) return rc;
       if ((rc = run_col(h, cr, QG_K_COL_REDUCE))) return rc;
       c.op = CO_DYN_COMBINE;
       c.nfwd = 0;
@@ -470,8 +479,7 @@ int enqueue_step(qg_handle* h) {
       c.op = CO_STAGE_STATIC;
       c.nfwd = h->nout;
       for (int i = 0; i < h->nout; ++i) c.fin[i] = h->Y[i];
-      c.stall_cta1 = h->inject_stall;
-      h->inject_stall = 0;
+      if ((rc = take_stall(h, c))) return rc;
     }
     if (s < 2) {
       c.store_ws = 1;

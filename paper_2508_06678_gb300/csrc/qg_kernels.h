@@ -142,6 +142,9 @@ template <typename T>
 cudaError_t launch_adj_germano_dots(const Geom& g, const void* H, const void* M, const AdjDotOut& o,
                                     cudaStream_t st);
 
+// Failure-handling test: a bounded wait that runs out and sets the status flag.
+cudaError_t launch_stall(int* err, cudaStream_t st);
+
 // Sets the thread-local message returned by qg_last_error().
 void set_last_error(const char* msg);
 
