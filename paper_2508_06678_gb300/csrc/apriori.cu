@@ -151,25 +151,29 @@ __global__ void moments_finish_kernel(const double* partials, int nblk, double* 
 }
 
 // A call's device memory, zeroed: blocks of 256-byte aligned size carved from one allocation of the size reserved
-// (a hundred allocations and frees of a call took longer than its kernels), others allocated as they are asked for.
+// (a hundred allocations and frees of a call took longer than its kernels), others allocated as they are asked for,
+// all of them where the reservation finds no room.
 struct Pool {
   std::vector<void*> ptrs;
   cudaError_t err = cudaSuccess;
   char* at = nullptr;
   size_t left = 0;
-  void reserve(size_t bytes) {
-    if (err != cudaSuccess) return;
+  static size_t size(size_t bytes) { return (bytes + 255) / 256 * 256; }
+  bool reserve(size_t bytes) {
     void* p = nullptr;
-    err = cudaMalloc(&p, bytes);
-    if (err != cudaSuccess) return;
+    if (cudaMalloc(&p, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
     cudaMemsetAsync(p, 0, bytes, nullptr);
     ptrs.push_back(p);
     at = static_cast<char*>(p);
     left = bytes;
+    return true;
   }
   void* get(size_t bytes) {
-    const size_t need = (bytes + 255) / 256 * 256;
-    if (need > left) reserve(need);
+    const size_t need = size(bytes);
+    if (err == cudaSuccess && need > left && !reserve(need)) err = cudaErrorMemoryAllocation;
     if (err != cudaSuccess) return nullptr;
     void* p = at;
     at += need;
@@ -208,6 +212,9 @@ struct Uploads {
     if (st) cudaStreamDestroy(st);
   }
 };
+
+// doubles of a call's partial sums, Germano results, and PCC moments
+constexpr size_t kPartials = 2 * 4096, kCoefs = 8, kMoments = 5 * 1024;
 
 struct Ctx {
   cudaStream_t st = nullptr;
@@ -282,11 +289,15 @@ extern "C" int qg_sgs_apriori(const double* omega_fr, int32_t n_fr, int32_t n_le
   Ctx cx;
   Uploads up;
   {
-    auto m = [](const Grid& G) { return (size_t)G.g.n * G.g.IP * 16 + 256; };
-    auto sp = [](const Grid& G) { return (size_t)G.g.Kcp * G.g.SP * 16 + 256; };
-    auto ph = [](int n) { return (size_t)n * n * 8 + 256; };
-    pool.reserve(10 * m(F) + 6 * sp(F) + 3 * ph(n_fr) + 18 * m(Cg) + m(Cf) + 14 * sp(Cg) + 2 * sp(Cf) + 7 * ph(n_les) +
-                 3 * (size_t)n_fr * 32 + (1u << 17));
+    // what is asked for below
+    auto m = [](const Grid& G) { return Pool::size((size_t)G.g.n * G.g.IP * 16); };
+    auto sp = [](const Grid& G) { return Pool::size((size_t)G.g.Kcp * G.g.SP * 16); };
+    auto ph = [](int n) { return Pool::size((size_t)n * n * 8); };
+    auto tab = [](const Grid& G) { return Pool::size(((size_t)G.plan.table * 2 + G.g.n / 2 + 1) * 8); };
+    const size_t opt = (mask_fr ? 1 : 0) + (sponge_fr ? 1 : 0);
+    pool.reserve(tab(F) + tab(Cg) + tab(Cf) + (1 + opt) * ph(n_fr) + 10 * m(F) + (2 + 2 * opt) * sp(F) + 18 * m(Cg) +
+                 m(Cf) + 14 * sp(Cg) + opt * sp(Cf) + (5 + opt) * ph(n_les) + Pool::size(kPartials * 8) +
+                 Pool::size(kCoefs * 8) + Pool::size(kMoments * 8));
   }
   auto mixed = [&](const Grid& G) { return pool.get((size_t)G.g.n * G.g.IP * 16); };
   auto spec = [&](const Grid& G) { return pool.get((size_t)G.g.Kcp * G.g.SP * 16); };
@@ -333,9 +344,9 @@ extern "C" int qg_sgs_apriori(const double* omega_fr, int32_t n_fr, int32_t n_le
   void* Pcchis = sponge_fr ? phys(n_les) : nullptr;
   void* Pout[5];
   for (int i = 0; i < 5; ++i) Pout[i] = phys(n_les);
-  double* partials = (double*)pool.get(2 * 4096 * sizeof(double));
-  double* coef = (double*)pool.get(8 * sizeof(double));
-  double* mom = (double*)pool.get(5 * 1024 * sizeof(double));
+  double* partials = (double*)pool.get(kPartials * 8);
+  double* coef = (double*)pool.get(kCoefs * 8);
+  double* mom = (double*)pool.get(kMoments * 8);
   if (pool.err != cudaSuccess) {
     qg::set_last_error("qg_sgs_apriori: device allocation failed");
     return QG_ERR_OOM;
