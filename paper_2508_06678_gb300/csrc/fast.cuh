@@ -30,7 +30,7 @@ template <typename T, int N> struct Eng {
                                               bool active) {
     if constexpr (I < P.np) {
       C* buf = ph ? b1 : b0;
-      st_pass<C, N, EL, I, PK, true>(x, t, buf, ptw, sign, active);
+      st_pass<C, N, EL, I, PK, true>(x, t, buf, ptw, sign, active, BUF, nullptr);
       if constexpr (I < P.np - 1) {
         __syncthreads();
 #pragma unroll

@@ -508,9 +508,11 @@ template <int EL_> struct RtShape {
 };
 
 // Pass I of the compile-time transform of length N: x in natural ownership on entry; a non-last pass writes its
-// outputs to buf (when active), the last one leaves them in x.
+// outputs to buf (when active; len elements, status bits st in the bounds-checked debug build), the last one leaves
+// them in x.
 template <typename C, int N, int EL, int I, bool PK, bool GL>
-__device__ __forceinline__ void st_pass(C* x, int t, C* buf, const C* tw, int s, bool active) {
+__device__ __forceinline__ void st_pass(C* x, int t, C* buf, const C* tw, int s, bool active, int len, int* st) {
+  (void)len; (void)st;
   constexpr Radices P = fft_radices(N, EL);
   constexpr int R = P.radix[I], NS = P.ns[I], NB = EL / R, TT = N / EL;
 #pragma unroll
@@ -528,7 +530,7 @@ __device__ __forceinline__ void st_pass(C* x, int t, C* buf, const C* tw, int s,
     } else if (active) {
       const int base = (j / NS) * NS * R + k;
 #pragma unroll
-      for (int r = 0; r < R; ++r) buf[fft_pad(base + NS * r)] = v[r];
+      for (int r = 0; r < R; ++r) QG_ST(buf, fft_pad(base + NS * r), len, st, v[r]);
     }
   }
 }
@@ -548,11 +550,11 @@ template <int N_, int EL_> struct StShape {
     if constexpr (I < np) {
       constexpr bool last = I == np - 1;
       C* buf = last ? nullptr : fb.take();
-      st_pass<C, N_, EL_, I, true, false>(x, t, buf, tw, -1, fb.active);
+      st_pass<C, N_, EL_, I, true, false>(x, t, buf, tw, -1, fb.active, fb.len, fb.st);
       if constexpr (!last) {
         fb.sync();
 #pragma unroll
-        for (int m = 0; m < EL; ++m) x[m] = buf[fft_pad(t + N_ / EL_ * m)];
+        for (int m = 0; m < EL; ++m) x[m] = QG_LD(buf, fft_pad(t + N_ / EL_ * m), fb.len, fb.st);
         from<I + 1>(x, t, fb, tw);
       }
     }
