@@ -4,8 +4,6 @@
 // per grid size.
 #pragma once
 
-#include <atomic>
-
 #include "fast.cuh"
 #include "qg_kernels.h"
 #include "spectral.cuh"
@@ -30,6 +28,8 @@
 namespace qg {
 namespace fast {
 
+constexpr int kBuildSms = 152;  // SMs of a GB300, where an occupancy has to be fixed at compile time
+
 template <int N> struct RowCfg {
   static constexpr int TT = Eng<float, N>::TT;
   // groups of TT threads, each with a row (or two rows that share a transform), filling at most QG_ROW_CTA_THREADS threads
@@ -50,7 +50,7 @@ template <int OP, int N> struct Occ {
   // The final passes take one CTA an SM, with more registers, where their column tiles need several rounds over the
   // SMs either way, and two where that makes it one round (dynamic Leith 1296^2 43.5 -> 38.3 us, 1536^2 49.7 -> 42.7)
   static constexpr int tiles = (Eng<float, N>::Kc + kFastWidth - 1) / kFastWidth;
-  static constexpr int fwd = tiles > 152 && tiles <= 304 && col_threads<N>() >= 192 ? 2 : QG_COL_MINB_FWD;
+  static constexpr int fwd = tiles > kBuildSms && tiles <= 2 * kBuildSms && col_threads<N>() >= 192 ? 2 : QG_COL_MINB_FWD;
   static constexpr int want = OP == CO_DYN_REDUCE ? QG_COL_MINB_REDUCE
                               : (OP == CO_FORWARD || OP == CO_FORWARD2 || OP == CO_FORWARD_N ||
                                  OP == CO_AB2CN_FINAL) ? fwd
@@ -1078,20 +1078,6 @@ cudaError_t launch_col_one(const Geom& g, const ColDesc& d, const cplx_t<T>* twp
   const cudaError_t e = raise_smem_limit<fast::col_fast_kernel<T, N, P, LEAN>>(smem);
   if (e != cudaSuccess) return e;
   return launch_pdl(d.pdl != 0, k, dim3(grid), dim3(Cfg::THREADS), smem, st, g, d, cs, twp, tm);
-}
-
-// SMs of the current device, queried once per device (concurrent first calls store the same value)
-inline int device_sms() {
-  static std::atomic<int> sms[64];
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev < 0 || dev >= 64) return 1;
-  int n = sms[dev].load(std::memory_order_relaxed);
-  if (!n) {
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 1;
-    sms[dev].store(n, std::memory_order_relaxed);
-  }
-  return n;
 }
 
 template <typename T, int N>

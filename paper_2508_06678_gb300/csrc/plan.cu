@@ -1,6 +1,7 @@
 // Host side of the run-time FFT engine (fft.cuh): plans, and the launch shapes of the passes that use it.
 #include "qg_kernels.h"
 
+#include <atomic>
 #include <cmath>
 #include <utility>
 
@@ -86,8 +87,20 @@ std::vector<double> fft_table(const FftPlan& p, int esz) {
   return t;
 }
 
+int device_sms() {
+  static std::atomic<int> sms[64];
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev < 0 || dev >= 64) return 1;
+  int n = sms[dev].load(std::memory_order_relaxed);
+  if (!n) {
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 1;
+    sms[dev].store(n, std::memory_order_relaxed);
+  }
+  return n;
+}
+
 // dynamic shared memory a CTA can have: 227 KB less the passes' static part (under 768 bytes)
-constexpr int kSms = 152;  // of a GB300
 constexpr size_t kSmemCap = 227 * 1024 - 768;
 
 static size_t tw_bytes(const FftPlan& p, int esz) { return tw_shared(p.table) ? (size_t)p.table * 2 * esz : 0; }
@@ -120,9 +133,9 @@ RowConfig row_config(const FftPlan& p, const RowDesc& d, int esz) {
   c.threads = (groups * p.tt + 31) / 32 * 32;
   // FP64 is bound by its operations, so the last, partial round of row pairs goes out as single rows where that
   // leaves no SM with two of them (1024^2: 3 pairs and a row per SM against 4 pairs)
-  const int pairs = p.n / c.rows, rest = pairs % kSms;
+  const int pairs = p.n / c.rows, sms = device_sms(), rest = pairs % sms;
   c.full = pairs;
-  if (esz == 8 && c.rows == 2 && !direct && pairs > kSms && rest > 0 && 2 * rest <= kSms) c.full = pairs - rest;
+  if (esz == 8 && c.rows == 2 && !direct && pairs > sms && rest > 0 && 2 * rest <= sms) c.full = pairs - rest;
   c.warp = p.tt <= 32 && 32 % p.tt == 0;
   return c;
 }
@@ -155,15 +168,15 @@ ColConfig col_config(const Geom& g, const FftPlan& p, const ColDesc& d, int W, i
   // at the price of transforming the incoming ones in each (1024^2: 342 columns, 38 of them in four parts; with the
   // single rows of row_config 1508 -> 1374 us per step).  Not with less than a round: 128^2, 43 columns in three
   // parts each, 140 us against 136.  Not where an op reads what it writes: a column's parts run at the same time.
-  const int tiles = g.Kcp / W, rest = tiles % kSms;
+  const int tiles = g.Kcp / W, sms = device_sms(), rest = tiles % sms;
   bool reads_own = d.op == CO_AB2CN || d.op == CO_AB2CN_COMBINE ||
                    ((d.op == CO_STAGE_STATIC || d.op == CO_DYN_COMBINE) && d.store_w0);
   for (int i = 0; i < d.nfwd; ++i)
     for (int q = 0; q < d.nder; ++q) reads_own = reads_own || d.fin[i] == d.dout[q];
   c.full = tiles;
   c.split = 1;
-  if (esz == 8 && !reads_own && d.nder > 1 && rest > 0 && tiles > kSms) {
-    const int s = kSms / rest < d.nder ? kSms / rest : d.nder;
+  if (esz == 8 && !reads_own && d.nder > 1 && rest > 0 && tiles > sms) {
+    const int s = sms / rest < d.nder ? sms / rest : d.nder;
     if (s > 1) {
       c.split = s;
       c.full = tiles - rest;

@@ -5,6 +5,9 @@
 
 namespace qg {
 
+// SMs of the current device, queried once per device (concurrent first calls store the same value)
+int device_sms();
+
 // Launch shape of the row pass: rows per CTA, groups (transforms side by side), physical rows kept in shared memory
 // per row (slots).
 // (the first `full` CTAs have `rows` rows, the others one)
