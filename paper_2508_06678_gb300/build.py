@@ -15,8 +15,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libqg.so")
-# the bounds-checked debug build (every shared and global access of the generic row and column passes and their
-# FFT is checked; an index outside its array sets a status bit reported as QG_ERR_BOUNDS): tests only
+# the bounds-checked debug build (every shared and global access of the row and column passes that run transforms side
+# by side is checked; an index outside its array sets a status bit reported as QG_ERR_BOUNDS): tests only
 CHECKED_DIR = os.path.join(HERE, "_build_checked")
 CHECKED_FLAGS = ("-DQG_CHECKED",)
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -15,7 +15,7 @@ namespace fast {
 
 template <typename T, int N> struct Eng {
   using C = cplx_t<T>;
-  static constexpr int EL = fft_elems(N, (int)sizeof(T));
+  static constexpr int EL = fft_elems(N);
   static constexpr int TT = N / EL;
   static constexpr Radices P = fft_radices(N, EL);
   static constexpr int NEX = P.np - 1;    // shared-memory exchanges of one transform

@@ -56,6 +56,9 @@ template <int OP, int N> struct Occ {
                                  OP == CO_AB2CN_FINAL) ? fwd
                               : OP == CO_CURL    ? QG_COL_MINB_CURL
                                                  : QG_COL_MINB;
+  // (Never fewer than 128 registers: compiled for two CTAs of 384 threads, at 80, the 2304^2 stage pass gave wrong
+  // static-closure columns, the same ones every time.  Its accesses and barriers do not depend on the register count and
+  // no cause was found in them, so a compiler fault is likely; the tests run every grid.)
   static constexpr int most = 512 / col_threads<N>() > 0 ? 512 / col_threads<N>() : 1;
   static constexpr int col = want < most ? want : most;
 };

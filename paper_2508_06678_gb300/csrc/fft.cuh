@@ -55,19 +55,20 @@ constexpr Radices fft_radices(int n, int el) {
   r.table = off > 0 ? off : 1;
   return r;
 }
-// Elements per thread.  FP64: four for n = 2^a -- on this GPU an FP64 instruction occupies its quarter of an SM for
-// 64 cycles, so a transform's time is its FP64 operations, spread over as many warps as possible.  FP32: eight up to
-// 512 (a grid with few rows has idle SMs, and half as many elements per thread halve the chain), sixteen above (one
-// exchange fewer).  Factors of 3: twelve or eighteen, whichever needs fewer passes.
-constexpr int fft_elems(int n, int esz) {
-  if (n % 3) return esz == 8 ? 4 : n <= 512 ? 8 : 16;
+// Elements per thread of the FP32 passes specialised for n: eight up to 512 (a grid with few rows has idle SMs, and
+// half as many elements per thread halve the chain), sixteen above (one exchange fewer).  Factors of 3, in any pass:
+// twelve or eighteen, whichever needs fewer passes.
+constexpr int fft_elems(int n) {
+  if (n % 3) return n <= 512 ? 8 : 16;
   const int a = fft_radices(n, 12).np, b = fft_radices(n, 18).np;
   return a && (!b || a <= b) ? 12 : 18;
 }
 
-// the same for the run-time passes: a 2^a grid of FP32 reals keeps eight (its larger grids have passes of their own),
-// and so does 4096 in FP64, where four would take more threads than a CTA has
-constexpr int rt_elems(int n, int esz) { return n % 3 ? (esz == 8 && n <= 2048 ? 4 : 8) : fft_elems(n, esz); }
+// The same for the run-time passes.  FP64, n = 2^a: four -- on this GPU an FP64 instruction occupies its quarter of an
+// SM for 64 cycles at best (spectral.cuh), so a transform's time is its FP64 operations, spread over as many warps as possible; eight
+// at 4096, where four would take more threads than a CTA has.  A 2^a grid of FP32 reals keeps eight (its larger grids
+// have passes of their own).
+constexpr int rt_elems(int n, int esz) { return n % 3 ? (esz == 8 && n <= 2048 ? 4 : 8) : fft_elems(n); }
 // most threads of a CTA of the run-time passes: twelve and eighteen FP64 elements need 168 registers a thread
 constexpr int pass_threads(int el, int esz) { return esz == 8 && el > 8 ? 384 : 512; }
 
@@ -493,7 +494,6 @@ template <int EL_> struct RtShape {
         case 8: if constexpr (EL % 8 == 0) pass<8>(x, t, ps, last, buf, tw, fb); break;
         case 9: if constexpr (EL % 9 == 0) pass<9>(x, t, ps, last, buf, tw, fb); break;
         case 12: if constexpr (EL % 12 == 0) pass<12>(x, t, ps, last, buf, tw, fb); break;
-        case 16: if constexpr (EL % 16 == 0) pass<16>(x, t, ps, last, buf, tw, fb); break;
         case 18: if constexpr (EL % 18 == 0) pass<18>(x, t, ps, last, buf, tw, fb); break;
       }
       if (!last) {

@@ -1821,7 +1821,7 @@ int qg_create(const qg_grid* grid, double beta, double U, const double* mask, co
     // 126, 2048^2 681 / 732; FP64 128^2 143 / 136, 256^2 223 / 262.
     h->step_pdl = n <= (h->fp32 ? 324 : 162) ? 1 : 0;
     h->adj_pdl = h->fp32 || h->step_pdl;  // FP64 256^2 adjoint step 1.55 ms without, 1.85 with; FP32 0.354 and 0.331
-    h->plan = fft_plan(n, h->fast || h->wide ? fft_elems(n, 4) : rt_elems(n, (int)h->esz));
+    h->plan = fft_plan(n, h->fast || h->wide ? fft_elems(n) : rt_elems(n, (int)h->esz));
     if (const char* inj = getenv("QG_INJECT_TMA_STALL")) h->inject_stall = atoi(inj) + 1;
     h->W = h->fast ? kFastWidth : col_width(h->plan, (int)h->esz);
     const size_t adj_slots = closure->kind == QG_NONE ? 4 : closure->kind == QG_LEITH || closure->kind == QG_DLEITH ? 6 : 8;

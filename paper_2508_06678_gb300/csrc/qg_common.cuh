@@ -225,10 +225,6 @@ struct ColDesc {
                        // mbarrier but issues no copy at all, so its bounded wait runs out with nothing in flight
 };
 
-// Per-thread accumulator of the Germano sums.  FP64 fields accumulate in
-// FP64; FP32 fields use error-free transformations (TwoProduct by FMA,
-// TwoSum) so the per-thread partial carries about twice FP32 precision
-// before it joins the FP64 cross-thread reduction.
 // Programmatic dependent launch.  A kernel launched by launch_pdl may be scheduled while the kernel before
 // it on the stream is still finishing: it first waits here, before any memory access, until that kernel has
 // completed and its writes are visible, then lets the next kernel be scheduled.  Launched without the
@@ -248,8 +244,8 @@ inline bool pdl_enabled() {
 }
 
 // k<<<grid, block, smem, st>>>(args...), with programmatic stream serialisation when pdl is set (k must call
-// pdl_enter() first).  The adjoint's chains of small launches gain from it; the forward step's graph measured
-// slower with it, so its launches leave it off.
+// pdl_enter() first).  Chains of launches of a few microseconds gain from it: the adjoint's, and a step's on small grids
+// (FP32 up to 324, FP64 up to 162); on larger grids the waiting CTAs take room from the running ones.
 template <typename... P, typename... A>
 cudaError_t launch_pdl(bool pdl, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
   cudaLaunchConfig_t cfg = {};
@@ -320,6 +316,10 @@ cudaError_t raise_smem_limit(size_t bytes) {
   return e;
 }
 
+// Per-thread accumulator of the Germano sums.  FP64 fields accumulate in
+// FP64; FP32 fields use error-free transformations (TwoProduct by FMA,
+// TwoSum) so the per-thread partial carries about twice FP32 precision
+// before it joins the FP64 cross-thread reduction.
 template <typename T> struct GermanoAcc;
 template <> struct GermanoAcc<double> {
   double s = 0.0;

@@ -1,10 +1,11 @@
 // What the column passes share: the op's scalars in the working precision, 1 / |k|^2, and the reductions of the
 // dynamic closures.
 //
-// On this GPU an FP64 instruction holds its quarter of an SM for 64 cycles, a conversion to or from FP64 included, so
-// the FP32 passes take their scalars ready converted, read 1 / |k|^2 of the smallest wavenumbers (inverted in FP64)
-// from a table, and keep the FP64 sums short: the two Germano sums share every instruction (one per half warp), and
-// all warps of a CTA add up the partial sums where one warp did.
+// On this GPU an FP64 instruction holds its quarter of an SM for 64 cycles at best (half a lane a cycle, 1.26 TFLOP/s;
+// chains of independent FMAs reach 1.06, one instruction in 76), a conversion to or from FP64 included, so the FP32
+// passes take their scalars ready converted, read 1 / |k|^2 of the smallest wavenumbers (inverted in FP64) from a table,
+// and keep the FP64 sums short: the two Germano sums share every instruction (one per half warp), and all warps of a
+// CTA add up the partial sums where one warp did.
 #pragma once
 
 #include <cmath>

@@ -9,12 +9,12 @@ namespace qg {
 
 template <int N>
 cudaError_t launch_row_wide(const Geom& g, const FftPlan& plan, const RowDesc& d, const void* tw, cudaStream_t st) {
-  return launch_row_shape<float>(g, plan, StShape<N, fft_elems(N, 4)>{}, d, tw, st);
+  return launch_row_shape<float>(g, plan, StShape<N, fft_elems(N)>{}, d, tw, st);
 }
 template <int N>
 cudaError_t launch_col_wide(const Geom& g, const FftPlan& plan, const ColDesc& d, const void* tw, int W,
                             cudaStream_t st) {
-  return launch_col_shape<float>(g, plan, StShape<N, fft_elems(N, 4)>{}, d, tw, W, st);
+  return launch_col_shape<float>(g, plan, StShape<N, fft_elems(N)>{}, d, tw, W, st);
 }
 
 #define QG_INSTANTIATE_WIDE(N)                                                                                    \
