@@ -280,6 +280,7 @@ extern "C" int qg_sgs_apriori(const double* omega_fr, int32_t n_fr, int32_t n_le
   int dev = 0, optin = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  // fine grids up to 3072 (the limit of a column pass of two columns, kept as this call's)
   if (2 * (size_t)n_fr * 16 + 4 * (size_t)F.g.Ny * 16 > (size_t)optin - 1024 || F.row_smem > (size_t)optin - 1024 || Cg.row_smem > (size_t)optin - 1024) {
     qg::set_last_error("qg_sgs_apriori: grid too large for the kernels' shared memory");
     return QG_ERR_UNSUPPORTED;
@@ -622,6 +623,7 @@ extern "C" int qg_grid_filter(const double* omega_fr, int32_t nsnap, int32_t n_f
   int dev = 0, optin = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  // fine grids up to 3072 (the limit of a column pass of two columns, kept as this call's)
   if (2 * (size_t)n_fr * 16 + 4 * (size_t)F.g.Ny * 16 > (size_t)optin - 1024 || F.row_smem > (size_t)optin - 1024) {
     qg::set_last_error("qg_grid_filter: grid too large for the kernels' shared memory");
     return QG_ERR_UNSUPPORTED;
